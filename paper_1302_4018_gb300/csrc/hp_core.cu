@@ -503,6 +503,102 @@ __global__ void k_probe_phases(LatGeom g, uint32_t first, int count, uint16_t* _
   }
 }
 
+// Phases of real vectors (hierarchical m < 2^K, or natural-order Hadamard): phase = (P/2) parity(val(site) & col(m)),
+// with val the binary part of loc (bit 31: the sign of z_0) and col(m) the bit reversal of m over K bits, or
+// val = site and col = m.
+// Bound by the 2-byte stores.  The entries of 8 consecutive vectors (m = 8 g .. 8 g + 7) differ only in the three bits
+// of val that the low bits of m select, so one population count per site and 8 vectors gives all 8 entries, kept as the
+// bits of a byte in shared memory; the block then writes its tile row by row in 16-byte stores (8 entries), shifting
+// the bytes to the alignment of each row (a ragged V puts every row at another offset).
+// 512 vectors of 64^3 with z_0 (268 MB): 593 us with one thread per entry (64-bit division, gather of loc, SplitMix64
+// and a modulo per entry) -> 37 us (7.2 TB/s written).
+constexpr int PT = 256, PTILE = 8 * PT;
+__global__ void __launch_bounds__(PT) k_probe_signs(LatGeom g, uint32_t first, uint32_t end, int groups_per_block,
+                                                    uint16_t* __restrict__ out) {
+  __shared__ __align__(16) unsigned char sh[2][PTILE + 16];
+  const int t0 = blockIdx.x * PTILE, nt = min(PTILE, g.V - t0);
+  const bool natural = g.probe_kind == HP_PROBE_NATURAL;
+  uint32_t val[8];
+  unsigned int walsh = 0, walsh_hi = 0;   // one byte per site of this thread: its entries' dependence on m & 7
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int i = threadIdx.x + k * PT;
+    val[k] = 0;
+    if (i >= nt) continue;
+    const uint32_t site = (uint32_t)(t0 + i);
+    uint32_t v = natural ? site : g.loc[site];
+    if (!natural && g.Q > 1) v /= (uint32_t)g.Q;
+    unsigned int w = 0;
+    for (int b = 0; b < 3 && b < g.K; ++b)
+      if ((v >> (natural ? b : g.K - 1 - b)) & 1u) w ^= b == 0 ? 0xAAu : b == 1 ? 0xCCu : 0xF0u;
+    if (k < 4) walsh |= w << (8 * k);
+    else walsh_hi |= w << (8 * (k - 4));
+    if (g.z0_seed && (splitmix64_at(g.z0_seed, site) >> 63)) v |= 0x80000000u;
+    val[k] = v;
+  }
+  const uint32_t half = (uint32_t)(g.P >> 1);
+  const uint32_t g0 = (first >> 3) + blockIdx.y * (uint32_t)groups_per_block;
+  const uint32_t g1 = min(g0 + (uint32_t)groups_per_block, (end + 7u) >> 3);
+  int buf = 0;
+  for (uint32_t gr = g0; gr < g1; ++gr, buf ^= 1) {
+    const uint32_t m0 = 8u * gr;
+    const uint32_t col = (natural ? m0 : (g.K > 0 ? __brev(m0) >> (32 - g.K) : 0u)) | 0x80000000u;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const unsigned int w = (k < 4 ? walsh >> (8 * k) : walsh_hi >> (8 * (k - 4))) & 0xffu;
+      sh[buf][threadIdx.x + k * PT] = (unsigned char)(w ^ ((__popc(val[k] & col) & 1) ? 0xffu : 0u));
+    }
+    __syncthreads();   // one barrier per group: the next group fills the other buffer
+#pragma unroll
+    for (uint32_t j = 0; j < 8; ++j) {
+      const uint32_t m = m0 + j;
+      if (m < first || m >= end) continue;
+      uint16_t* row = out + (size_t)(m - first) * g.V + t0;
+      const int head = min(nt, (int)((0u - (unsigned int)((uintptr_t)row >> 1)) & 7u));   // entries before a 16-byte boundary
+      const int nv = (nt - head) >> 3, v = threadIdx.x;
+      if (v < nv) {
+        const int i = head + 8 * v;
+        const unsigned int* wp = reinterpret_cast<const unsigned int*>(sh[buf] + (i & ~3));
+        const unsigned int s8 = 8u * (i & 3), a = wp[0], b = wp[1], c = wp[2];
+        const unsigned int lo = (__funnelshift_r(a, b, s8) >> j) & 0x01010101u;
+        const unsigned int hi = (__funnelshift_r(b, c, s8) >> j) & 0x01010101u;
+        *reinterpret_cast<uint4*>(row + i) =
+            make_uint4(__byte_perm(lo, 0, 0x4140) * half, __byte_perm(lo, 0, 0x4342) * half,
+                       __byte_perm(hi, 0, 0x4140) * half, __byte_perm(hi, 0, 0x4342) * half);
+      }
+      const int rest = nt - 8 * nv;   // < 16: the head and the tail
+      if (v < rest) {
+        const int i = v < head ? v : v + 8 * nv;
+        row[i] = (uint16_t)(((sh[buf][i] >> j) & 1u) * half);
+      }
+    }
+  }
+}
+
+// Z_2 noise: entry (m, site) takes output number m V + site of SplitMix64, so the vectors are one run of outputs and
+// the entries are generated in the order they lie in memory, 8 to a 16-byte store.
+__global__ void __launch_bounds__(PT) k_probe_z2(unsigned long long seed, unsigned long long index0, size_t n, uint32_t half,
+                                                 uint16_t* __restrict__ out) {
+  const size_t head0 = (0u - (unsigned int)((uintptr_t)out >> 1)) & 7u;
+  const size_t head = head0 < n ? head0 : n, nv = (n - head) >> 3, stride = (size_t)gridDim.x * PT;
+  const size_t t = (size_t)blockIdx.x * PT + threadIdx.x;
+  for (size_t v = t; v < nv; v += stride) {
+    const size_t i = head + 8 * v;
+    unsigned int w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const unsigned int a = (unsigned int)(splitmix64_at(seed, index0 + i + 2 * k) >> 63);
+      const unsigned int b = (unsigned int)(splitmix64_at(seed, index0 + i + 2 * k + 1) >> 63);
+      w[k] = (a | b << 16) * half;
+    }
+    *reinterpret_cast<uint4*>(out + i) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+  if (t < n - 8 * nv) {
+    const size_t i = t < head ? t : t + 8 * nv;
+    out[i] = (uint16_t)((unsigned int)(splitmix64_at(seed, index0 + i) >> 63) * half);
+  }
+}
+
 static int grid_for(hp_ctx* ctx, long long n, int threads) {
   long long b = (n + threads - 1) / threads;
   long long cap = (long long)ctx->num_sms * 16;
@@ -629,10 +725,35 @@ extern "C" hp_status hp_probe_sequence(hp_ctx* ctx, const hp_lattice* lat, int32
   LatGeom g = ls->g;
   g.z0_seed = z0_seed;
   g.probe_kind = kind;
-  {
+  if (kind == HP_PROBE_Z2) {
+    const size_t n = (size_t)count * g.V;
+    ProfScope ps(ctx, "k_probe_z2");
+    k_probe_z2<<<grid_for(ctx, (long long)(n / 8 + 8), PT), PT, 0, ctx->stream>>>(
+        z0_seed, (unsigned long long)first * (unsigned long long)g.V, n, (uint32_t)(g.P >> 1), phase_dev);
+    HP_LAUNCH_CHECK();
+    return HP_OK;
+  }
+  // vectors with real entries: those of natural order, the hierarchical ones of the binary levels
+  const int64_t n_real = kind == HP_PROBE_NATURAL ? (int64_t)g.V : (int64_t)1 << g.K;
+  const int64_t end = first + count, real_end = std::min(end, n_real);
+  if (first < real_end) {
+    const int tiles = (g.V + PTILE - 1) / PTILE;
+    const int64_t groups = ((real_end + 7) >> 3) - (first >> 3);
+    // groups of 8 vectors per block: a tile's site data serve as many groups as leave four blocks per SM (and fit
+    // the grid)
+    int64_t gy = std::max<int64_t>(1, std::min<int64_t>(groups, ((int64_t)ctx->num_sms * 4 + tiles - 1) / tiles));
+    const int64_t per = (groups + gy - 1) / gy;
+    gy = (groups + per - 1) / per;
+    ProfScope ps(ctx, "k_probe_signs");
+    k_probe_signs<<<dim3(tiles, (unsigned)gy), PT, 0, ctx->stream>>>(g, (uint32_t)first, (uint32_t)real_end, (int)per,
+                                                                     phase_dev);
+    HP_LAUNCH_CHECK();
+  }
+  if (end > n_real) {   // the three-colour and Fourier levels
+    const int64_t f2 = std::max(first, n_real);
     ProfScope ps(ctx, "k_probe_phases");
-    k_probe_phases<<<grid_for(ctx, count * (long long)g.V, 256), 256, 0, ctx->stream>>>(g, (uint32_t)first,
-                                                                                          (int)count, phase_dev);
+    k_probe_phases<<<grid_for(ctx, (end - f2) * (long long)g.V, 256), 256, 0, ctx->stream>>>(
+        g, (uint32_t)f2, (int)(end - f2), phase_dev + (size_t)(f2 - first) * g.V);
   }
   HP_LAUNCH_CHECK();
   return HP_OK;

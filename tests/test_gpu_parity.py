@@ -70,6 +70,26 @@ def test_permutation_full_size_sampled(ctx, dims):
     assert np.array_equal(l[sites], np.array(P.hierarchical_loc(dims, sites)))
 
 
+# tiles of 2048 sites, rows at every offset to 16 bytes, groups of 8 vectors cut at both ends, a range across the
+# binary and the Fourier levels
+@pytest.mark.parametrize("dims,kind,first,count,shift", [
+    ((64, 32), "hp", 3, 14, 0), ((64, 33), "hp", 0, 64, 0), ((6, 6, 6, 10), "hp", 5, 11, 1), ((2049,), "hp", 0, 1, 3),
+    ((12, 6, 5, 7), "hp", 1, 7, 0), ((6, 6, 6, 6), "hp", 10, 20, 5), ((2,), "hp", 0, 2, 0), ((64, 64), "natural", 7, 18, 2),
+    ((2, 2), "natural", 0, 4, 0), ((45, 46), "z2", 3, 5, 7), ((3,), "z2", 0, 2, 1)])
+def test_probe_rows_at_every_alignment(ctx, hp, dims, kind, first, count, shift):
+    V = int(np.prod(dims))
+    buf = torch.full((count * V + 16,), 7, dtype=torch.int16, device="cuda:0")
+    per = ctx.probe_vectors(dims, first, count, 2003, buf[shift:shift + count * V], kind=kind)
+    if kind == "hp":
+        ref, P = Pr.probe_phases(dims, first, count, 2003)
+    else:
+        P = hp.basis_info(dims)["period"]
+        ref = (Pr.probe_phases_natural if kind == "natural" else Pr.probe_phases_z2)(V, first, count, 2003) * (P // 2)
+    got = buf.cpu().numpy().astype(np.int64) & 0xFFFF
+    assert per == P and np.array_equal(got[shift:shift + count * V].reshape(count, V), ref)
+    assert (got[:shift] == 7).all() and (got[shift + count * V:] == 7).all()
+
+
 @pytest.mark.parametrize("dims,seed", [((4, 4), 0), ((2, 4, 8), 5), ((4, 4, 4, 4), 2003), ((6, 6, 6, 6), 9),
                                        ((3, 3, 3, 3), 1), ((12, 6), 0), ((5, 4), 3), ((6, 2, 6, 2), 4)])
 def test_probe_phases_bit_exact(ctx, hp, dims, seed):
