@@ -616,6 +616,20 @@ def test_clover_gradient_vs_oracle(ctx, hp):
     assert np.allclose(g, g_ref, rtol=1e-7, atol=1e-9)
 
 
+# the masked launches (group and exact steps) spread the slots over blocks in classes: one class, several,
+# and more slots in a class than the block has threads
+@pytest.mark.parametrize("dims,s,block,prec", [((4, 4, 4, 4), 12, 4, "fp16"), ((4, 4, 4, 4), 12, 144, "fp32"),
+                                               ((8, 4, 4, 6), 2, 24, "fp64"), ((8, 8, 4, 4), 700, 8400, "fp16")])
+def test_masked_launches_serve_every_slot(ctx, hp, dims, s, block, prec):
+    U = synth.gauge_links(dims, 0.3, 77)
+    op = ctx.make_operator(hp.OP_WILSON, 0.0, 0.12, links_dev(U), None)
+    T, _, st = ctx.trace_inv(op, dims, s, 1e-10, ctx.make_opts(prec, rhs_block=block, z0_seed=5, even_odd=1))
+    assert st["rhs_solved"] == 12 * s and st["n_unconverged"] == 0 and st["max_true_residual"] <= 1e-10
+    T_ref = E.trace_prefix(E.wilson_quadratures(dims, U, 0.12, 0, min(s, 2), 5, method="dense")) if s < 100 else \
+        ctx.trace_inv(op, dims, s, 1e-10, ctx.make_opts("fp64", rhs_block=64, z0_seed=5))[0]
+    assert np.all(rel(T[:len(T_ref)], T_ref) <= TRACE_RTOL)
+
+
 # ------------------------------------------------------------------ the comparison sequences (Section 5.2)
 @pytest.mark.parametrize("kind,dims,seed", [("natural", (8, 8, 8, 8), 0), ("natural", (2, 4, 8), 11),
                                             ("natural", (1024,), 3), ("z2", (4, 4, 4, 4), 12345),
