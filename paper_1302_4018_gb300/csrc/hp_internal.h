@@ -346,7 +346,9 @@ __device__ __forceinline__ bool last_block(unsigned int* counter, unsigned int n
   return am_last != 0;
 }
 
-// sum of partials[q][0..nparts) in a fixed order by one block; result in every thread's out[q]
+// sum of partials[q][0..nparts) in a fixed order by one block; result in every thread's out[q].
+// One warp adds the NT per-thread sums (FP64 runs at 2 lanes per clock, and the step is a serial chain that every
+// launch waits for: one barrier instead of a tree of them).
 template <int NQ, int NTHREADS>
 __device__ __forceinline__ void block_sum_partials(const double* part, size_t q_stride, int nparts, double (&out)[NQ]) {
   __shared__ double sh2[NQ][NTHREADS];
@@ -357,13 +359,18 @@ __device__ __forceinline__ void block_sum_partials(const double* part, size_t q_
     sh2[q][threadIdx.x] = t;
   }
   __syncthreads();
-  for (int s = NTHREADS / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
+  if (threadIdx.x < 32) {
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) sh2[q][threadIdx.x] += sh2[q][threadIdx.x + s];
+    for (int q = 0; q < NQ; ++q) {
+      double t = 0.0;
+#pragma unroll
+      for (int w = 0; w < NTHREADS / 32; w += 2) t += sh2[q][threadIdx.x + 32 * w] + sh2[q][threadIdx.x + 32 * w + 32];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+      if (threadIdx.x == 0) sh2[q][0] = t;
     }
-    __syncthreads();
   }
+  __syncthreads();
 #pragma unroll
   for (int q = 0; q < NQ; ++q) out[q] = sh2[q][0];
   __syncthreads();

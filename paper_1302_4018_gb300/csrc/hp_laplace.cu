@@ -16,34 +16,45 @@ static int lblocks(hp_ctx* ctx, long long n, int threads) {
   return (int)std::max(1LL, std::min(b, cap));
 }
 
-__device__ __forceinline__ double lap_site(const LatGeom& g, const double* __restrict__ x, int site) {
-  if (g.csr_rp) {   // a general sparse matrix: row `site` of A times x
-    double acc = 0.0;
-    for (int e = g.csr_rp[site]; e < g.csr_rp[site + 1]; ++e) acc += g.csr_val[e] * __ldg(x + g.csr_ci[e]);
-    return acc;
-  }
+// The diagonal as the stencil below uses it: 8 + m + mu(s), less 2 for every extent of 1 (there both neighbours are the
+// site itself).  FP64 adds bound the stencil (2 lanes per clock and SM), so a 3-D lattice padded to four dimensions does
+// not add its own site twice.
+__device__ __forceinline__ double lap_diag0(const LatGeom& g) {
+  double d = 8.0 + g.mass;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (g.L[j] == 1) d -= 2.0;
+  return d;
+}
+
+template <bool MF>   // MF: a per-site mass field (a branch per site would add it on the FP64 pipe either way)
+__device__ __forceinline__ double lap_site(const LatGeom& g, double diag0, const double* __restrict__ x, int site) {
   int r = site, st = 1;
   double acc = 0.0;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int L = g.L[j];
+    if (L == 1) continue;   // uniform over the grid
     const int xj = r % L;
     r /= L;
     const int fw = (xj + 1 == L) ? site - (L - 1) * st : site + st;
     const int bw = (xj == 0) ? site + (L - 1) * st : site - st;
-    acc += __ldg(x + fw) + __ldg(x + bw);
+    const double t = __ldg(x + fw) + __ldg(x + bw);
+    acc = j == 0 ? t : acc + t;
     st *= L;
   }
-  const double diag = 8.0 + g.mass + (g.mass_field ? g.mass_field[site] : 0.0);
-  return diag * __ldg(x + site) - acc;
+  const double diag = MF ? diag0 + g.mass_field[site] : diag0;
+  return fma(diag, __ldg(x + site), -acc);
 }
 
 __global__ void k_lap_apply(LatGeom g, const double* __restrict__ in, double* __restrict__ out, int nrhs) {
   const long long total = (long long)nrhs * g.V;
+  const double diag0 = lap_diag0(g);
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
     int rhs = (int)(t / g.V), site = (int)(t - (long long)rhs * g.V);
-    out[t] = lap_site(g, in + (size_t)rhs * g.V, site);
+    const double* x = in + (size_t)rhs * g.V;
+    out[t] = g.mass_field ? lap_site<true>(g, diag0, x, site) : lap_site<false>(g, diag0, x, site);
   }
 }
 
@@ -80,14 +91,12 @@ struct LArgs {
   double *x, *r, *p, *q;   // [slot][Vmax]
   double tol2;
   int maxiter;
-  int by_slot;   // 1: grid (tiles, slots), 0: grid (slots, tiles)
+  int nslots;
   double* dc;    // deflation: V^T b of each slot's source, [slot][defl_k]
 };
 
 #define LSLOT(COND)                                                \
-  const int slot = a.by_slot ? blockIdx.y : blockIdx.x;            \
-  const int bx = a.by_slot ? blockIdx.x : blockIdx.y;              \
-  const int gx = a.by_slot ? gridDim.x : gridDim.y;                \
+  const int slot = blockIdx.x, bx = blockIdx.y, gx = gridDim.y;    \
   SlotState* S = a.st + slot;                                      \
   if (!(COND)) return;                                             \
   const LatGeom g = a.lats[S->lat];                                \
@@ -138,24 +147,24 @@ __global__ void __launch_bounds__(NT) k_cg_defl(LArgs a) {
   }
 }
 
+// Block sum of v into part[q * gy + bx].  One warp adds the block's values (NT / 32 per lane, then a shuffle tree):
+// NT / 32 + 5 FP64 warp instructions a block, where a shuffle tree in every warp takes 5 NT / 32 and FP64 runs at 2
+// lanes per clock (8^4, 256 slots: see k_cg_xr).
 template <int NQ, int NT>
 __device__ __forceinline__ void lreduce(double (&v)[NQ], double* part, int gy, int bx) {
-  __shared__ double sh[NQ][NT / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double sh[NQ][NT];
 #pragma unroll
-  for (int qq = 0; qq < NQ; ++qq) {
-    double t = v[qq];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) sh[qq][warp] = t;
-  }
+  for (int qq = 0; qq < NQ; ++qq) sh[qq][threadIdx.x] = v[qq];
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {
 #pragma unroll
     for (int qq = 0; qq < NQ; ++qq) {
       double t = 0.0;
-      for (int w = 0; w < NT / 32; ++w) t += sh[qq][w];
-      part[(size_t)qq * gy + bx] = t;
+#pragma unroll
+      for (int w = 0; w < NT / 32; w += 2) t += sh[qq][threadIdx.x + 32 * w] + sh[qq][threadIdx.x + 32 * w + 32];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+      if (threadIdx.x == 0) part[(size_t)qq * gy + bx] = t;
     }
   }
 }
@@ -258,18 +267,38 @@ __global__ void __launch_bounds__(NT) k_cg_init(LArgs a) {
   }
 }
 
-// q = A p ; alpha = rr / (p, q)
+// Sites of a block: tiles bx, bx + gx, ..., U of them per step, so that a thread has U independent sets of loads (and
+// of FP64 chains) in flight.
+#define LTILES(U) for (int tile = bx; tile < ntiles; tile += (U) * gx)
+#define LSITE(u) const int site = (tile + (u) * gx) * NT + (int)threadIdx.x
+
+// q = A p ; alpha = rr / (p, q).  Bound by the FP64 pipe (5 or 7 adds, 2 FMAs a site: 47 us for 16 slots of 64^3).
+template <int NT, bool MF>
+__device__ __forceinline__ double cg_ap_sites(const LatGeom& g, const double* __restrict__ p, double* __restrict__ q,
+                                              int bx, int gx, int ntiles) {
+  const double diag0 = lap_diag0(g);
+  double acc = 0.0;
+  LTILES(2) {
+    double qv[2], pv[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      LSITE(u);
+      qv[u] = pv[u] = 0.0;
+      if (site >= g.V) continue;
+      qv[u] = lap_site<MF>(g, diag0, p, site);
+      pv[u] = __ldg(p + site);
+      q[site] = qv[u];
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) acc = fma(pv[u], qv[u], acc);
+  }
+  return acc;
+}
 template <int NT>
 __global__ void __launch_bounds__(NT) k_cg_ap(LArgs a) {
   LSLOT(S->status == SLOT_RUN)
-  double acc[1] = {0.0};
-  for (int tile = bx; tile < ntiles; tile += gx) {
-    const int site = tile * NT + threadIdx.x;
-    if (site >= g.V) continue;
-    double qv = lap_site(g, a.p + off, site);
-    a.q[off + site] = qv;
-    acc[0] += a.p[off + site] * qv;
-  }
+  double acc[1] = {g.mass_field ? cg_ap_sites<NT, true>(g, a.p + off, a.q + off, bx, gx, ntiles)
+                                : cg_ap_sites<NT, false>(g, a.p + off, a.q + off, bx, gx, ntiles)};
   lreduce<1, NT>(acc, part, a.gy, bx);
   if (last_block(a.cnt + slot, nparts)) {
     double tot[1];
@@ -287,13 +316,30 @@ __global__ void __launch_bounds__(NT) k_cg_xr(LArgs a) {
   LSLOT(S->status == SLOT_RUN)
   const double al = S->alpha.x;
   double acc[1] = {0.0};
-  for (int tile = bx; tile < ntiles; tile += gx) {
-    const int site = tile * NT + threadIdx.x;
-    if (site >= g.V) continue;
-    a.x[off + site] += al * a.p[off + site];
-    double rv = a.r[off + site] - al * a.q[off + site];
-    a.r[off + site] = rv;
-    acc[0] += rv * rv;
+  double* __restrict__ x = a.x + off;
+  double* __restrict__ r = a.r + off;
+  const double* __restrict__ p = a.p + off;
+  const double* __restrict__ q = a.q + off;
+  LTILES(2) {
+    double xv[2], pv[2], rv[2], qv[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      LSITE(u);
+      if (site >= g.V) continue;
+      xv[u] = x[site];
+      pv[u] = p[site];
+      rv[u] = r[site];
+      qv[u] = q[site];
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      LSITE(u);
+      if (site >= g.V) continue;
+      x[site] = fma(al, pv[u], xv[u]);
+      const double rn = fma(-al, qv[u], rv[u]);
+      r[site] = rn;
+      acc[0] = fma(rn, rn, acc[0]);
+    }
   }
   lreduce<1, NT>(acc, part, a.gy, bx);
   if (last_block(a.cnt + slot, nparts)) {
@@ -306,27 +352,51 @@ __global__ void __launch_bounds__(NT) k_cg_xr(LArgs a) {
   }
 }
 
-// true residual r = b - A x
+// true residual r = b - A x.  Most iterations no slot asks for one: the grid is (1, tiles, classes) and block z
+// loops over the slots z, z + gz, ... that ask (a slot is finalised by the last block that serves it, so all of them
+// read its flag before); a block per (slot, tile) cost 10-12 us per idle launch.
 template <int NT>
 __global__ void __launch_bounds__(NT) k_cg_true(LArgs a) {
-  LSLOT(S->need_update)
-  double acc[1] = {0.0};
-  const int m = S->m, pa = S->a;
-  for (int tile = bx; tile < ntiles; tile += gx) {
-    const int site = tile * NT + threadIdx.x;
-    if (site >= g.V) continue;
-    double rv = lap_src(g, a, slot, site, m, pa) - lap_site(g, a.x + off, site);
-    a.r[off + site] = rv;
-    acc[0] += rv * rv;
-  }
-  lreduce<1, NT>(acc, part, a.gy, bx);
-  if (last_block(a.cnt + slot, nparts)) {
-    double tot[1];
-    block_sum_partials<1, NT>(part, a.gy, nparts, tot);
-    if (threadIdx.x == 0) {
-      cg_after_true(S, tot[0], a.tol2);
-      a.cnt[slot] = 0;
+  __shared__ unsigned int want;
+  // the flags of up to 32 of the block's slots at a time, one per lane
+  for (int s0 = blockIdx.z; s0 < a.nslots; s0 += 32 * gridDim.z) {
+   __syncthreads();
+   if (threadIdx.x < 32) {
+    const int sl = s0 + (int)threadIdx.x * gridDim.z;
+    const unsigned int b = __ballot_sync(0xffffffffu, sl < a.nslots && a.st[min(sl, a.nslots - 1)].need_update);
+    if (threadIdx.x == 0) want = b;
+   }
+   __syncthreads();
+   for (unsigned int todo = want; todo; todo &= todo - 1) {
+    const int slot = s0 + (__ffs(todo) - 1) * gridDim.z;
+    SlotState* S = a.st + slot;
+    const LatGeom g = a.lats[S->lat];
+    const int ntiles = (g.V + NT - 1) / NT, bx = blockIdx.y, gx = gridDim.y;
+    if (bx >= ntiles) continue;
+    const int nparts = min(gx, ntiles);
+    double* part = a.part + (size_t)slot * 4 * a.gy;
+    const size_t off = (size_t)slot * a.Vmax;
+    const double diag0 = lap_diag0(g);
+    double acc[1] = {0.0};
+    const int m = S->m, pa = S->a;
+    for (int tile = bx; tile < ntiles; tile += gx) {
+      const int site = tile * NT + threadIdx.x;
+      if (site >= g.V) continue;
+      const double ax = g.mass_field ? lap_site<true>(g, diag0, a.x + off, site) : lap_site<false>(g, diag0, a.x + off, site);
+      const double rv = lap_src(g, a, slot, site, m, pa) - ax;
+      a.r[off + site] = rv;
+      acc[0] += rv * rv;
     }
+    lreduce<1, NT>(acc, part, a.gy, bx);
+    if (last_block(a.cnt + slot, nparts)) {
+      double tot[1];
+      block_sum_partials<1, NT>(part, a.gy, nparts, tot);
+      if (threadIdx.x == 0) {
+        cg_after_true(S, tot[0], a.tol2);
+        a.cnt[slot] = 0;
+      }
+    }
+   }
   }
 }
 
@@ -334,10 +404,22 @@ template <int NT>
 __global__ void __launch_bounds__(NT) k_cg_p(LArgs a) {
   LSLOT(S->status == SLOT_RUN)
   const double be = S->restart ? 0.0 : S->beta.x;
-  for (int tile = bx; tile < ntiles; tile += gx) {
-    const int site = tile * NT + threadIdx.x;
-    if (site >= g.V) continue;
-    a.p[off + site] = a.r[off + site] + be * a.p[off + site];
+  double* __restrict__ p = a.p + off;
+  const double* __restrict__ r = a.r + off;
+  LTILES(4) {
+    double pv[4], rv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      LSITE(u);
+      if (site >= g.V) continue;
+      pv[u] = p[site];
+      rv[u] = r[site];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      LSITE(u);
+      if (site < g.V) p[site] = fma(be, pv[u], rv[u]);
+    }
   }
 }
 
@@ -378,20 +460,16 @@ __global__ void k_lgrad(LArgs a, int lat, const int* __restrict__ slots, int nsl
 
 struct LaplaceEngine {
   static constexpr int NT = 256;
+  static constexpr int LAP_BLOCKS = 6;   // resident blocks per SM
   int kernels_per_iteration() const { return 4; }
   static constexpr int GROUP_MAX = 1;
   hp_ctx* ctx;
   LArgs a;
-  int nslots, gy;
+  int nslots, gy, gy_true, gz_true;
   int big_lat = 0;   // index of the largest lattice (set by the scheduler; unused here)
   bool one_lat = false;   // one lattice in the problem (set by the scheduler; unused here)
   int defl_k = 0;
-  // A sparse matrix runs with slots along y: the blocks of one slot are scheduled together,
-  // so the vector its rows gather from stays in L2 while the slot runs (slots along x would
-  // interleave all of them, and every gather of a renumbered matrix would be a DRAM sector).
-  // The lattice stencil reads neighbours that are near in memory; there slots along x measured
-  // faster (all slots stream at once).
-  dim3 grid() const { return a.by_slot ? dim3(gy, nslots) : dim3(nslots, gy); }
+  dim3 grid() const { return dim3(nslots, gy); }
   int group() const { return 1; }
   hp_status setup(int ns, int Vmax, const LatGeom* lats_dev, SlotState* st, const hp_solver_opts& o, double tol,
                   double, const LatGeom& big) {
@@ -400,11 +478,16 @@ struct LaplaceEngine {
     a.lats = lats_dev;
     a.st = st;
     a.Vmax = Vmax;
-    int ntiles = (Vmax + NT - 1) / NT;
-    gy = std::max(1, std::min(std::min(ntiles, ctx->num_sms * 4), 65535));
-    a.gy = gy;
+    a.nslots = ns;
+    // one resident wave over all slots: a thread then sums several sites before the block's FP64 shuffle sums (ten
+    // adds per warp, as much as the stencil of one site) and a slot has few partial sums
+    const int ntiles = (Vmax + NT - 1) / NT;
+    gy = std::max(1, std::min(ntiles, (ctx->num_sms * LAP_BLOCKS + ns - 1) / ns));
+    gy_true = std::max(1, std::min(ntiles, ctx->num_sms * 2));
+    gz_true = std::max(1, std::min({ns, ctx->num_sms * LAP_BLOCKS / gy_true, 64}));
+    a.gy = std::max(gy, gy_true);
     void* p = nullptr;
-    HP_TRY(hp_ws(ctx, "solve.part", sizeof(double) * 4 * (size_t)ns * gy, &p));
+    HP_TRY(hp_ws(ctx, "solve.part", sizeof(double) * 4 * (size_t)ns * a.gy, &p));
     a.part = (double*)p;
     HP_TRY(hp_ws(ctx, "solve.cnt", sizeof(unsigned int) * ns, &p));
     a.cnt = (unsigned int*)p;
@@ -420,7 +503,6 @@ struct LaplaceEngine {
     a.q = (double*)p;
     a.tol2 = tol * tol;
     a.maxiter = o.maxiter > 0 ? o.maxiter : 10000;
-    a.by_slot = big.csr_rp != nullptr;
     defl_k = big.defl_k;
     if (defl_k) {
       HP_TRY(hp_ws(ctx, "solve.defl_c", sizeof(double) * (size_t)ns * defl_k, &p));
@@ -443,7 +525,7 @@ struct LaplaceEngine {
   hp_status iteration() {
     { ProfScope ps(ctx, "k_cg_ap"); k_cg_ap<NT><<<grid(), NT, 0, ctx->stream>>>(a); }
     { ProfScope ps(ctx, "k_cg_xr"); k_cg_xr<NT><<<grid(), NT, 0, ctx->stream>>>(a); }
-    { ProfScope ps(ctx, "k_cg_true"); k_cg_true<NT><<<grid(), NT, 0, ctx->stream>>>(a); }
+    { ProfScope ps(ctx, "k_cg_true"); k_cg_true<NT><<<dim3(1, gy_true, gz_true), NT, 0, ctx->stream>>>(a); }
     { ProfScope ps(ctx, "k_cg_p"); k_cg_p<NT><<<grid(), NT, 0, ctx->stream>>>(a); }
     HP_LAUNCH_CHECK();
     return HP_OK;
@@ -1186,7 +1268,7 @@ static hp_status run_blocked(hp_ctx* ctx, SolveProblem& pb, SolveResult& res) {
 }
 
 hp_status hp_solve_laplace(hp_ctx* ctx, SolveProblem& pb, SolveResult& res) {
-  if (pb.lats.size() == 1 && pb.lats[0].csr_rp && !pb.want_grad) {
+  if (pb.lats[0].csr_rp) {   // a general sparse matrix (always alone, without a gradient)
     // blocked engine: B slots (rhs_block rounded up to 32, 64 or 128; automatic: 64, the fastest
     // on the renumbered 64^3 grid matrix in both precisions)
     const int want = pb.opts.rhs_block > 0 ? pb.opts.rhs_block : 64;
