@@ -470,6 +470,7 @@ struct LaplaceEngine {
   bool one_lat = false;   // one lattice in the problem (set by the scheduler; unused here)
   int defl_k = 0;
   dim3 grid() const { return dim3(nslots, gy); }
+  static size_t slot_bytes(const LaplaceEngine&, int Vmax) { return 32 * (size_t)Vmax; }
   int group() const { return 1; }
   hp_status setup(int ns, int Vmax, const LatGeom* lats_dev, SlotState* st, const hp_solver_opts& o, double tol,
                   double, const LatGeom& big) {
@@ -1141,6 +1142,7 @@ struct BlockedSparseEngine {
   long long nnz = 0;
   double delta = 0.0;
   int group() const { return 1; }
+  static size_t slot_bytes(const BlockedSparseEngine&, int Vmax) { return 32 * (size_t)Vmax; }   // rhs_block is always set
   hp_status setup(int ns, int Vmax, const LatGeom* lats_dev, SlotState* st, const hp_solver_opts& o, double tol,
                   double, const LatGeom&) {
     if (ns != B) {

@@ -34,10 +34,28 @@ hp_status run_schedule(hp_ctx* ctx, Engine& eng, SolveProblem& pb, SolveResult& 
     for (int64_t m = pb.first[L]; m < pb.s_max[L]; ++m)
       for (int a = 0; a < dof; ++a) queue.push_back({L, (int)m, a});
   }
+  // Automatic slot count: up to 256 slots, all of the queue at once where its vectors fit 8 GB and half of the memory
+  // that is free (or already held for them), else 4M sites' worth.  More slots mean fewer and larger launches: an uneven
+  // batch (168 right-hand sides of 8^4, 12^4, 16^3x32) took 47.8 ms in 32 slots, 40.4 in 96, 39.8 in 168 (whose 11 GB
+  // cost a first call more than that); 96 of 16^4 45.4 ms in 64, 43.4 in 96; 24 of 32^3x64 328 ms in 12, 326 in 24.
+  // Rounds of equal size: 300 right-hand sides run as 2 x 150.
   int nslots = pb.opts.rhs_block;
-  if (nslots <= 0) {
-    long long want = (4LL << 20) / std::max(1, Vmax);
-    nslots = (int)std::max(12LL, std::min(want, 256LL));
+  const bool automatic = nslots <= 0;
+  const int small_slots = (int)std::max(12LL, std::min((4LL << 20) / std::max(1, Vmax), 256LL));
+  if (automatic) {
+    nslots = small_slots;
+    const size_t per = Engine::slot_bytes(eng, Vmax);
+    const long long fit = (long long)((8ULL << 30) / std::max<size_t>(1, per));
+    long long want = std::min<long long>({(long long)queue.size(), 256LL, fit});
+    if (want > nslots) {
+      size_t free_b = 0, total_b = 0, held = 0;
+      HP_CUDA(cudaMemGetInfo(&free_b, &total_b));
+      for (auto& kv : ctx->ws)
+        if (kv.first.compare(0, 6, "solve.") == 0) held += kv.second.bytes;
+      if (per * (size_t)want <= (free_b + held) / 2) nslots = (int)want;
+    }
+    const long long rounds = ((long long)queue.size() + nslots - 1) / nslots;
+    if (rounds > 1 && nslots > small_slots) nslots = (int)(((long long)queue.size() + rounds - 1) / rounds);
   }
   nslots = (int)std::min<long long>(nslots, std::max<size_t>(1, queue.size()));
   nslots = std::min(nslots, 65535);   // one grid dimension of the solver kernels
@@ -58,7 +76,13 @@ hp_status run_schedule(hp_ctx* ctx, Engine& eng, SolveProblem& pb, SolveResult& 
   memset(host.data(), 0, sizeof(SlotState) * nslots);
   eng.big_lat = big;
   eng.one_lat = nl == 1;
-  HP_TRY(eng.setup(nslots, Vmax, lats_dev, st_dev, pb.opts, pb.tol, delta, pb.lats[big]));
+  hp_status su = eng.setup(nslots, Vmax, lats_dev, st_dev, pb.opts, pb.tol, delta, pb.lats[big]);
+  if (su == HP_ENOMEM && automatic && nslots > small_slots) {   // fragmented memory: the smaller slot count
+    nslots = (small_slots + Engine::GROUP_MAX - 1) / Engine::GROUP_MAX * Engine::GROUP_MAX;
+    host.resize(nslots);
+    su = eng.setup(nslots, Vmax, lats_dev, st_dev, pb.opts, pb.tol, delta, pb.lats[big]);
+  }
+  HP_TRY(su);
   const int G = eng.group();   // slots refilled together (one lattice per group: the stencil shares links)
 
   const int chunk = pb.opts.check_every > 0 ? pb.opts.check_every : 8;

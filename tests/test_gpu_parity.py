@@ -630,6 +630,31 @@ def test_masked_launches_serve_every_slot(ctx, hp, dims, s, block, prec):
     assert np.all(rel(T[:len(T_ref)], T_ref) <= TRACE_RTOL)
 
 
+# the prefix kernel works 256 probes at a time: one, the edges of a chunk, several chunks; it sums in order
+@pytest.mark.parametrize("s", [1, 255, 256, 257, 1000])
+def test_trace_prefix_chunks(ctx, s):
+    rng = np.random.default_rng(s)
+    q = rng.standard_normal(s) + 1j * rng.standard_normal(s)
+    T = ctx.trace_prefix(q)
+    acc, ref = 0j, []
+    for m in range(s):
+        acc += q[m]
+        ref.append(complex(acc.real / (m + 1), acc.imag / (m + 1)))
+    assert np.array_equal(T, np.array(ref))
+
+
+# the CG kernels take two sites per thread and step, skip extents of 1 and add the two neighbours of an extent of 2
+@pytest.mark.parametrize("dims,s,mf", [((1, 1, 5, 1), 1, 0), ((2, 1, 2, 2), 4, 1), ((2, 2, 2, 2), 16, 0), ((257,), 1, 1),
+                                       ((16, 33), 8, 0), ((6, 5, 4, 3), 8, 1), ((8, 8, 4, 2), 300, 0)])
+def test_laplacian_trace_ragged_extents(ctx, hp, dims, s, mf):
+    mu = np.abs(synth.mass_field(dims, 0.3, 9)) if mf else None
+    op = ctx.make_operator(hp.OP_LAPLACIAN, 0.2, mass_field=None if mu is None else dev(mu))
+    T, _, st = ctx.trace_inv(op, dims, s, 1e-12, ctx.make_opts("fp64", z0_seed=4, probe_kind="z2"))
+    assert st["max_true_residual"] <= 1e-12 and st["n_unconverged"] == 0
+    T_ref = E.trace_prefix(E.laplacian_quadratures(dims, 0.2, 0, s, 4, method="dense", kind="z2", mass_field=mu))
+    assert np.all(rel(T, T_ref) <= TRACE_RTOL)
+
+
 # ------------------------------------------------------------------ the comparison sequences (Section 5.2)
 @pytest.mark.parametrize("kind,dims,seed", [("natural", (8, 8, 8, 8), 0), ("natural", (2, 4, 8), 11),
                                             ("natural", (1024,), 3), ("z2", (4, 4, 4, 4), 12345),
