@@ -655,6 +655,26 @@ def test_laplacian_trace_ragged_extents(ctx, hp, dims, s, mf):
     assert np.all(rel(T, T_ref) <= TRACE_RTOL)
 
 
+# the direct FP64 application: odd volumes (a warp's last lanes idle), extents of 1 and 2, blocks of 64 and 128
+# threads, and an output that overlaps the input (served by the staged path); rounding: 200 terms of FP64 per site
+@pytest.mark.parametrize("dims,nrhs,mf", [((1, 1, 1, 1), 1, 0), ((3, 1, 2, 1), 5, 1), ((7, 5, 3, 3), 2, 0), ((5,), 1, 1),
+                                          ((2, 2, 2, 2), 3, 1), ((16, 9, 8, 7), 11, 1)])
+def test_wilson_apply_fp64_direct_and_in_place(ctx, hp, dims, nrhs, mf):
+    V = int(np.prod(dims))
+    pad = tuple(dims) + (1,) * (4 - len(dims))
+    U = synth.gauge_links(pad, 0.4, 31)
+    psi = synth.random_spinors(pad, nrhs, 32)
+    mu = synth.mass_field(pad, 0.1, 33) if mf else None
+    op = ctx.make_operator(hp.OP_WILSON, 0.05, 0.13, links_dev(U), None if mu is None else dev(mu))
+    x = dev(psi.reshape(nrhs, V, 12))
+    y = torch.empty_like(x)
+    ctx.operator_apply(op, dims, nrhs, "fp64", x, y)
+    ref = np.stack([O.wilson_apply(psi[i], U, pad, 0.13, 0.05, mu).reshape(V, 12) for i in range(nrhs)])
+    assert np.abs(y.cpu().numpy() - ref).max() <= 200 * 2.3e-16 * np.abs(ref).max()
+    ctx.operator_apply(op, dims, nrhs, "fp64", x, x)
+    assert np.abs(x.cpu().numpy() - ref).max() <= 200 * 2.3e-16 * np.abs(ref).max()
+
+
 # ------------------------------------------------------------------ the comparison sequences (Section 5.2)
 @pytest.mark.parametrize("kind,dims,seed", [("natural", (8, 8, 8, 8), 0), ("natural", (2, 4, 8), 11),
                                             ("natural", (1024,), 3), ("z2", (4, 4, 4, 4), 12345),
