@@ -496,17 +496,13 @@ __device__ __forceinline__ void reduce_pair(const float (&v)[2][NQ], double* par
       if (lane == 0) sh[L][q][warp] = (double)t;
     }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 2 * NQ) {   // one thread per lane and quantity
+    const int L = threadIdx.x / NQ, q = threadIdx.x % NQ;
+    if (L == 0 || two) {
+      double t = 0.0;
 #pragma unroll
-    for (int L = 0; L < 2; ++L) {
-      if (L == 1 && !two) break;
-      double* part = L ? part_b : part_a;
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        double t = 0.0;
-        for (int w = 0; w < NT / 32; ++w) t += sh[L][q][w];
-        part[(size_t)q * gy + blockIdx.y] = t;
-      }
+      for (int w = 0; w < NT / 32; ++w) t += sh[L][q][w];
+      (L ? part_b : part_a)[(size_t)q * gy + blockIdx.y] = t;
     }
   }
 }

@@ -120,7 +120,6 @@ __device__ __forceinline__ double2 dmul(double2 a, double2 b) {
 
 template <typename R, int NQ, int NT>
 __device__ __forceinline__ void reduce_partials(R (&v)[NQ], double* part, int gy) {
-  double dv[NQ];
   // warp level in the iteration precision, across warps in FP64
   __shared__ double sh[NQ][NT / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -132,14 +131,11 @@ __device__ __forceinline__ void reduce_partials(R (&v)[NQ], double* part, int gy
     if (lane == 0) sh[q][warp] = (double)t;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < NQ) {   // one thread per quantity: NT / 32 FP64 warp instructions a block, not NQ NT / 32
+    double t = 0.0;
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      double t = 0.0;
-      for (int w = 0; w < NT / 32; ++w) t += sh[q][w];
-      dv[q] = t;
-      part[(size_t)q * gy + blockIdx.y] = t;
-    }
+    for (int w = 0; w < NT / 32; ++w) t += sh[threadIdx.x][w];
+    part[(size_t)threadIdx.x * gy + blockIdx.y] = t;
   }
 }
 
@@ -444,6 +440,15 @@ __global__ void __launch_bounds__(NT) k_bicg_init(WArgs a) {
   }
 }
 
+// The vector updates of FP64 fields walk a site's components a few at a time (a chunk is one component): with all twelve
+// of every field in registers they took 168-255 registers, two blocks per SM.
+__device__ __forceinline__ const double2* comp64(FieldPtr f, int Vmax, int slot, int site) {
+  return (const double2*)f.p + (size_t)slot * 12 * Vmax + site;
+}
+__device__ __forceinline__ double2* comp64w(FieldPtr f, int Vmax, int slot, int site) {
+  return (double2*)f.p + (size_t)slot * 12 * Vmax + site;
+}
+
 // ---- s = r - alpha v
 template <int SPR, int NT>
 __global__ void __launch_bounds__(NT) k_bicg_s(WArgs a) {
@@ -454,13 +459,23 @@ __global__ void __launch_bounds__(NT) k_bicg_s(WArgs a) {
   for (int tile = blockIdx.y; tile < ntiles; tile += gridDim.y) {
     const int site = tile * NT + threadIdx.x;
     if (site >= nsite) continue;
+    if constexpr (SPR == PR64) {
+      const double2 *pr = comp64(a.r, a.Vmax, slot, site), *pv = comp64(a.v, a.Vmax, slot, site);
+      double2* ps = comp64w(a.s, a.Vmax, slot, site);
+#pragma unroll 6
+      for (int k = 0; k < 12; ++k) {
+        const double2 r = __ldg(pr + (size_t)k * a.Vmax), v = __ldg(pv + (size_t)k * a.Vmax);
+        ps[(size_t)k * a.Vmax] = make_double2(fma(ay, v.y, fma(-ax, v.x, r.x)), fma(-ay, v.x, fma(-ax, v.y, r.y)));
+      }
+      continue;
+    }
     cplx<R> r[12], v[12];
     SpinorIO<SPR>::load(a.r, a.Vmax, slot, site, r);
     SpinorIO<SPR>::load(a.v, a.Vmax, slot, site, v);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      r[k].x -= ax * v[k].x - ay * v[k].y;
-      r[k].y -= ax * v[k].y + ay * v[k].x;
+      r[k].x = fma(ay, v[k].y, fma(-ax, v[k].x, r[k].x));
+      r[k].y = fma(-ay, v[k].x, fma(-ax, v[k].y, r[k].y));
     }
     SpinorIO<SPR>::store(a.s, a.Vmax, slot, site, r);
   }
@@ -471,12 +486,33 @@ template <int SPR, int EPR, int NT>
 __global__ void __launch_bounds__(NT) k_bicg_xr(WArgs a) {
   SLOT_PREAMBLE(S->status == SLOT_RUN)
   typedef typename Real_of<SPR>::T R;
-  typedef typename Real_of<EPR>::T RE;
-  const double2 al = S->alpha, om = S->omega;
+  typedef R RE;
+  static_assert(SPR == EPR, "the solution increment is kept in the iteration precision");
+  // plain chains of FMAs: two per complex multiply-add and real part, where a product subtracted from a product costs a
+  // third operation (FP64 vectors are bound by the FP64 pipe: 12^4, 12 slots, xr 85 -> 58, p 45 -> 30, s 28 -> 18 us)
+  const R ax = (R)S->alpha.x, ay = (R)S->alpha.y, ox = (R)S->omega.x, oy = (R)S->omega.y;
   R acc[3] = {0, 0, 0};
   for (int tile = blockIdx.y; tile < ntiles; tile += gridDim.y) {
     const int site = tile * NT + threadIdx.x;
     if (site >= nsite) continue;
+    if constexpr (SPR == PR64) {
+      const double2 *pp = comp64(a.p, a.Vmax, slot, site), *ps = comp64(a.s, a.Vmax, slot, site),
+                    *pt = comp64(a.t, a.Vmax, slot, site), *ph = comp64(a.rh, a.Vmax, slot, site);
+      double2 *pe = comp64w(a.e, a.Vmax, slot, site), *pr = comp64w(a.r, a.Vmax, slot, site);
+#pragma unroll 4
+      for (int k = 0; k < 12; ++k) {
+        const size_t o = (size_t)k * a.Vmax;
+        const double2 p = __ldg(pp + o), sv = __ldg(ps + o), t = __ldg(pt + o), h = __ldg(ph + o), e = pe[o];
+        pe[o] = make_double2(fma(ax, p.x, fma(-ay, p.y, fma(ox, sv.x, fma(-oy, sv.y, e.x)))),
+                             fma(ax, p.y, fma(ay, p.x, fma(ox, sv.y, fma(oy, sv.x, e.y)))));
+        const double rx = fma(oy, t.y, fma(-ox, t.x, sv.x)), ry = fma(-oy, t.x, fma(-ox, t.y, sv.y));
+        pr[o] = make_double2(rx, ry);
+        acc[0] = fma(h.x, rx, fma(h.y, ry, acc[0]));
+        acc[1] = fma(h.x, ry, fma(-h.y, rx, acc[1]));
+        acc[2] = fma(rx, rx, fma(ry, ry, acc[2]));
+      }
+      continue;
+    }
     cplx<R> p[12], s[12], t[12], rh[12];
     cplx<RE> e[12];
     SpinorIO<SPR>::load(a.p, a.Vmax, slot, site, p);
@@ -486,13 +522,11 @@ __global__ void __launch_bounds__(NT) k_bicg_xr(WArgs a) {
     SpinorIO<EPR>::load(a.e, a.Vmax, slot, site, e);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      RE px = (RE)p[k].x, py = (RE)p[k].y, sx = (RE)s[k].x, sy = (RE)s[k].y;
-      e[k].x += (RE)al.x * px - (RE)al.y * py + (RE)om.x * sx - (RE)om.y * sy;
-      e[k].y += (RE)al.x * py + (RE)al.y * px + (RE)om.x * sy + (RE)om.y * sx;
-      cplx<R> rn;
-      rn.x = s[k].x - ((R)om.x * t[k].x - (R)om.y * t[k].y);
-      rn.y = s[k].y - ((R)om.x * t[k].y + (R)om.y * t[k].x);
-      s[k] = rn;
+      const RE px = (RE)p[k].x, py = (RE)p[k].y, sx = (RE)s[k].x, sy = (RE)s[k].y;
+      e[k].x = fma(ax, px, fma(-ay, py, fma(ox, sx, fma(-oy, sy, e[k].x))));
+      e[k].y = fma(ax, py, fma(ay, px, fma(ox, sy, fma(oy, sx, e[k].y))));
+      s[k].x = fma(oy, t[k].y, fma(-ox, t[k].x, s[k].x));
+      s[k].y = fma(-oy, t[k].x, fma(-ox, t[k].y, s[k].y));
     }
     SpinorIO<EPR>::store(a.e, a.Vmax, slot, site, e);
     SpinorIO<SPR>::store(a.r, a.Vmax, slot, site, s);
@@ -500,10 +534,9 @@ __global__ void __launch_bounds__(NT) k_bicg_xr(WArgs a) {
     if (SPR == PR16 || SPR == PRB16) SpinorIO<SPR>::load(a.r, a.Vmax, slot, site, s);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      cplx<R> d = cconjmul(rh[k], s[k]);
-      acc[0] += d.x;
-      acc[1] += d.y;
-      acc[2] += s[k].x * s[k].x + s[k].y * s[k].y;
+      acc[0] = fma(rh[k].x, s[k].x, fma(rh[k].y, s[k].y, acc[0]));
+      acc[1] = fma(rh[k].x, s[k].y, fma(-rh[k].y, s[k].x, acc[1]));
+      acc[2] = fma(s[k].x, s[k].x, fma(s[k].y, s[k].y, acc[2]));
     }
   }
   reduce_partials<R, 3, NT>(acc, part, a.gy);
@@ -734,6 +767,23 @@ __global__ void __launch_bounds__(NT) k_bicg_p(WArgs a) {
   for (int tile = blockIdx.y; tile < ntiles; tile += gridDim.y) {
     const int site = tile * NT + threadIdx.x;
     if (site >= nsite) continue;
+    if constexpr (SPR == PR64) {
+      const double2 *pr = comp64(a.r, a.Vmax, slot, site), *pv = comp64(a.v, a.Vmax, slot, site);
+      double2 *pp = comp64w(a.p, a.Vmax, slot, site), *ph = comp64w(a.rh, a.Vmax, slot, site);
+#pragma unroll 4
+      for (int k = 0; k < 12; ++k) {
+        const size_t o = (size_t)k * a.Vmax;
+        const double2 r = __ldg(pr + o);
+        if (restart) {
+          pp[o] = ph[o] = r;
+          continue;
+        }
+        const double2 p = pp[o], v = __ldg(pv + o);
+        const double dx = fma(oy, v.y, fma(-ox, v.x, p.x)), dy = fma(-oy, v.x, fma(-ox, v.y, p.y));
+        pp[o] = make_double2(fma(bx, dx, fma(-by, dy, r.x)), fma(bx, dy, fma(by, dx, r.y)));
+      }
+      continue;
+    }
     cplx<R> r[12], p[12], v[12];
     SpinorIO<SPR>::load(a.r, a.Vmax, slot, site, r);
     if (restart) {
@@ -745,10 +795,10 @@ __global__ void __launch_bounds__(NT) k_bicg_p(WArgs a) {
     SpinorIO<SPR>::load(a.v, a.Vmax, slot, site, v);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      R dx = p[k].x - (ox * v[k].x - oy * v[k].y);
-      R dy = p[k].y - (ox * v[k].y + oy * v[k].x);
-      p[k].x = r[k].x + (bx * dx - by * dy);
-      p[k].y = r[k].y + (bx * dy + by * dx);
+      const R dx = fma(oy, v[k].y, fma(-ox, v[k].x, p[k].x));
+      const R dy = fma(-oy, v[k].x, fma(-ox, v[k].y, p[k].y));
+      p[k].x = fma(bx, dx, fma(-by, dy, r[k].x));
+      p[k].y = fma(bx, dy, fma(by, dx, r[k].y));
     }
     SpinorIO<SPR>::store(a.p, a.Vmax, slot, site, p);
   }
@@ -1037,18 +1087,16 @@ __global__ void __launch_bounds__(NT, EO_ODD_MINB(SIN, REC)) k_eo_odd(WArgs a, F
       SpinorIO<SIN>::load(a.rh, a.Vmax, slot, h, rh);
 #pragma unroll
       for (int k = 0; k < 12; ++k) {
-        cplx<R> d = cconjmul(rh[k], acc[k]);
-        dots[0] += d.x;
-        dots[1] += d.y;
+        dots[0] = fma(rh[k].x, acc[k].x, fma(rh[k].y, acc[k].y, dots[0]));
+        dots[1] = fma(rh[k].x, acc[k].y, fma(-rh[k].y, acc[k].x, dots[1]));
       }
     } else {
       R d0 = 0, d1 = 0;
 #pragma unroll
       for (int k = 0; k < 12; ++k) {
-        cplx<R> d = cconjmul(acc[k], c[k]);
-        d0 += d.x;
-        d1 += d.y;
-        dots[2 % NQ] += acc[k].x * acc[k].x + acc[k].y * acc[k].y;
+        d0 = fma(acc[k].x, c[k].x, fma(acc[k].y, c[k].y, d0));
+        d1 = fma(acc[k].x, c[k].y, fma(-acc[k].y, c[k].x, d1));
+        dots[2 % NQ] = fma(acc[k].x, acc[k].x, fma(acc[k].y, acc[k].y, dots[2 % NQ]));
       }
       dots[0] += nc * d0;
       dots[1] += nc * d1;
