@@ -27,8 +27,11 @@ __device__ __forceinline__ double lap_diag0(const LatGeom& g) {
   return d;
 }
 
-template <bool MF>   // MF: a per-site mass field (a branch per site would add it on the FP64 pipe either way)
-__device__ __forceinline__ double lap_site(const LatGeom& g, double diag0, const double* __restrict__ x, int site) {
+// MF: a per-site mass field (a branch per site would add it on the FP64 pipe either way); NC: x is not written while the
+// kernel runs (read-only loads)
+template <bool MF, bool NC = true>
+__device__ __forceinline__ double lap_site(const LatGeom& g, double diag0, const double* x, int site) {
+  auto ld = [x](int i) { return NC ? __ldg(x + i) : x[i]; };
   int r = site, st = 1;
   double acc = 0.0;
 #pragma unroll
@@ -39,12 +42,12 @@ __device__ __forceinline__ double lap_site(const LatGeom& g, double diag0, const
     r /= L;
     const int fw = (xj + 1 == L) ? site - (L - 1) * st : site + st;
     const int bw = (xj == 0) ? site + (L - 1) * st : site - st;
-    const double t = __ldg(x + fw) + __ldg(x + bw);
+    const double t = ld(fw) + ld(bw);
     acc = j == 0 ? t : acc + t;
     st *= L;
   }
   const double diag = MF ? diag0 + g.mass_field[site] : diag0;
-  return fma(diag, __ldg(x + site), -acc);
+  return fma(diag, ld(site), -acc);
 }
 
 __global__ void k_lap_apply(LatGeom g, const double* __restrict__ in, double* __restrict__ out, int nrhs) {
@@ -470,7 +473,8 @@ struct LaplaceEngine {
   bool one_lat = false;   // one lattice in the problem (set by the scheduler; unused here)
   int defl_k = 0;
   dim3 grid() const { return dim3(nslots, gy); }
-  static size_t slot_bytes(const LaplaceEngine&, int Vmax) { return 32 * (size_t)Vmax; }
+  // keeps the scheduler at 4M sites' worth of slots: 128^2x64 with 32 vectors took 116 ms in 12 slots, 122 in 32
+  static size_t slot_bytes(const LaplaceEngine&, int) { return (size_t)8 << 30; }
   int group() const { return 1; }
   hp_status setup(int ns, int Vmax, const LatGeom* lats_dev, SlotState* st, const hp_solver_opts& o, double tol,
                   double, const LatGeom& big) {
@@ -1263,6 +1267,303 @@ struct BlockedSparseEngine {
 
 #include "hp_schedule.cuh"
 
+// ------------------------------------------------------------------ one right-hand side per cluster
+// A whole CG solve in one launch: a cluster of C thread blocks (C = 1, 2, 4, 8) owns one right-hand side, from the source to
+// the quadrature.  The launches of the slot engine cost about 10 us each in dependent latencies (flags, block
+// sums through L2, the scalar step), four of them an iteration, whatever the size; here a step ends in a cluster
+// barrier, the block sums travel through distributed shared memory, and every block takes the scalar steps on its own
+// copy of the state (the same sums in the same order, so all blocks agree on every branch and meet at every barrier).
+// The vectors stay in global memory (L2), read with plain loads: other blocks of the cluster write them.
+// Bound by the FP64 pipe (13 operations a site and iteration).
+// 8^4, 256 vectors: 2746 -> 1472 us; 64^3, 32 vectors: 30.8 -> 24.0 ms.
+__device__ __forceinline__ void cluster_barrier(int C) {
+  if (C == 1) {
+    __syncthreads();
+  } else {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  }
+}
+
+template <int CLT>
+struct ClusterSum {
+  double sh[CLT];
+  double in[2][8];   // the blocks' sums, two generations: a generation is read before the barrier after the next one's
+};
+// the cluster's sum of v in thread 0 of every block (other threads: undefined); a cluster barrier
+template <int CLT>
+__device__ __forceinline__ double cluster_sum(ClusterSum<CLT>& cs, double v, int C, int rank, int& gen) {
+  cs.sh[threadIdx.x] = v;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < CLT / 32; w += 2) t += cs.sh[threadIdx.x + 32 * w] + cs.sh[threadIdx.x + 32 * w + 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x < C) {
+      const unsigned int mine = (unsigned int)__cvta_generic_to_shared(&cs.in[gen][rank]);
+      unsigned int there;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(mine), "r"((unsigned int)threadIdx.x));
+      asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there), "d"(t) : "memory");
+    }
+  }
+  cluster_barrier(C);
+  double tot = 0.0;
+  if (threadIdx.x == 0)
+    for (int c = 0; c < C; ++c) tot += cs.in[gen][c];
+  gen ^= 1;
+  return tot;
+}
+
+template <bool MF, int CLT>
+__device__ __forceinline__ void cg_cluster_solve(const LArgs& a, const LatGeom& g, SlotState& S, ClusterSum<CLT>& cs, int item,
+                                                 double* x, double* r, double* p, double* q, int C, int rank, int most) {
+  const int lo = (int)((long long)g.V * rank / C), hi = (int)((long long)g.V * (rank + 1) / C);
+  const int m = S.m, pa = S.a;
+  const double diag0 = lap_diag0(g);
+  int gen = 0;
+  double acc = 0.0, tot;
+  if (S.status == SLOT_INIT) {
+    for (int i = lo + threadIdx.x; i < hi; i += CLT) {
+      const double b = lap_src(g, a, item, i, m, pa);
+      x[i] = 0.0;
+      r[i] = b;
+      p[i] = b;
+      acc = fma(b, b, acc);
+    }
+    tot = cluster_sum(cs, acc, C, rank, gen);
+    if (threadIdx.x == 0) cg_after_init(&S, g, tot);
+    __syncthreads();
+  }
+  // at most `most` iterations a launch; x, r, p and the state carry over to the next
+  for (int it = 0; S.status == SLOT_RUN && it < most; ++it) {
+    acc = 0.0;
+    for (int i = lo + threadIdx.x; i < hi; i += 2 * CLT) {
+      const int j = i + CLT;
+      const double q0 = lap_site<MF, false>(g, diag0, p, i), q1 = j < hi ? lap_site<MF, false>(g, diag0, p, j) : 0.0;
+      q[i] = q0;
+      acc = fma(p[i], q0, acc);
+      if (j < hi) {
+        q[j] = q1;
+        acc = fma(p[j], q1, acc);
+      }
+    }
+    tot = cluster_sum(cs, acc, C, rank, gen);
+    if (threadIdx.x == 0) cg_after_ap(&S, tot);
+    __syncthreads();
+    const double al = S.alpha.x;
+    acc = 0.0;
+    for (int i = lo + threadIdx.x; i < hi; i += 2 * CLT) {
+      const int j = i + CLT < hi ? i + CLT : i;
+      const double x0 = x[i], p0 = p[i], r0 = r[i], q0 = q[i], x1 = x[j], p1 = p[j], r1 = r[j], q1 = q[j];
+      const double n0 = fma(-al, q0, r0), n1 = fma(-al, q1, r1);
+      x[i] = fma(al, p0, x0);
+      r[i] = n0;
+      acc = fma(n0, n0, acc);
+      if (j != i) {
+        x[j] = fma(al, p1, x1);
+        r[j] = n1;
+        acc = fma(n1, n1, acc);
+      }
+    }
+    tot = cluster_sum(cs, acc, C, rank, gen);
+    if (threadIdx.x == 0) cg_after_xr(&S, g, tot, a.tol2, a.maxiter);
+    __syncthreads();
+    if (S.need_update) {   // the true residual r = b - A x
+      acc = 0.0;
+      for (int i = lo + threadIdx.x; i < hi; i += CLT) {
+        const double rv = lap_src(g, a, item, i, m, pa) - lap_site<MF, false>(g, diag0, x, i);
+        r[i] = rv;
+        acc = fma(rv, rv, acc);
+      }
+      tot = cluster_sum(cs, acc, C, rank, gen);
+      if (threadIdx.x == 0) cg_after_true(&S, tot, a.tol2);
+      __syncthreads();
+    }
+    if (S.status != SLOT_RUN) break;
+    const double be = S.restart ? 0.0 : S.beta.x;
+    for (int i = lo + threadIdx.x; i < hi; i += 2 * CLT) {
+      const int j = i + CLT < hi ? i + CLT : i;
+      const double p0 = p[i], r0 = r[i], p1 = p[j], r1 = r[j];
+      p[i] = fma(be, p0, r0);
+      if (j != i) p[j] = fma(be, p1, r1);
+    }
+    cluster_barrier(C);   // the next product reads the neighbours' p
+  }
+  if (S.status == SLOT_RUN) return;
+  acc = 0.0;
+  for (int i = lo + threadIdx.x; i < hi; i += CLT) acc = fma(lap_src(g, a, item, i, m, pa), x[i], acc);
+  tot = cluster_sum(cs, acc, C, rank, gen);   // no block leaves before the others have written their sums to it
+  if (threadIdx.x == 0) S.q = make_double2(tot, 0.0);
+}
+
+// item = first + number of the cluster; the vectors of an item of the launch at its number times Vmax.  (Vectors in
+// shared memory, one block of 131 KB per SM, measured slower than two blocks with the vectors in L2: 8^4, 256 vectors 1.66
+// against 1.47 ms.)
+template <int CLT>
+__global__ void __launch_bounds__(CLT, 1024 / CLT) k_cg_cluster(LArgs a, int first, int C, int most) {
+  __shared__ SlotState S;
+  __shared__ ClusterSum<CLT> cs;
+  const int cid = blockIdx.x / C, rank = blockIdx.x - cid * C, item = first + cid;
+  if (threadIdx.x == 0) S = a.st[item];
+  __syncthreads();
+  if (S.status != SLOT_INIT && S.status != SLOT_RUN) return;   // finished in an earlier launch (the whole cluster)
+  const LatGeom g = a.lats[S.lat];
+  const size_t off = (size_t)cid * a.Vmax;
+  if (C > 1) cluster_barrier(C);   // every block of the cluster has started: its shared memory can be written
+  if (g.mass_field) cg_cluster_solve<true, CLT>(a, g, S, cs, item, a.x + off, a.r + off, a.p + off, a.q + off, C, rank, most);
+  else cg_cluster_solve<false, CLT>(a, g, S, cs, item, a.x + off, a.r + off, a.p + off, a.q + off, C, rank, most);
+  __syncthreads();
+  if (threadIdx.x == 0 && rank == 0) a.st[item] = S;
+}
+
+// How a problem of n right-hand sides of V sites (on average) runs: C blocks of `threads` per right-hand side; C = 0: the
+// slot engine.
+struct ClusterPlan {
+  int C, threads;
+  int most;   // iterations per launch: about a second's worth at the most (a solve that needs more is launched again)
+};
+// The cost of an iteration over all right-hand sides in SM cycles: FP64 (6.5 cycles a site at 2 lanes per clock, at 0.8 of
+// the rate; at half of it where a block is alone on its SM with more than L1 holds of its vectors) on the busiest SM
+// plus the barriers, against the slot engine's FP64 over all SMs (0.7 of the rate) plus the latencies of its four
+// launches.  At equal cost the larger cluster: two blocks of 512 threads share an SM and fill each other's waits; blocks
+// that are alone on theirs take 1024 threads.  Both sides measured (clusters / slots): 64^3 with 32 vectors 24.0 / 30.8
+// ms, 16 23.4 / 15.0, 64 58.5 / 60; 32^3 with 2 1.9 / 2.8, 64 5.6 / 8.0; 8^4 with 1 0.51 / 1.1, 64 0.55 / 1.75.
+static ClusterPlan cluster_plan(const hp_ctx* ctx, double n, double V) {
+  ClusterPlan pl = {0, 512, 0};
+  double best = 1.4 * n * V * 6.5 / ctx->num_sms + 60e3;
+  for (int C = 1; C <= 8; C *= 2) {
+    if (C > 1 && V < 1024.0 * C) break;
+    const double k = std::ceil(n * C / ctx->num_sms);   // blocks on the busiest SM
+    const double cost = (k == 1.0 && V / C > 8192.0 ? 1.9 : 1.25 * k) * V * 6.5 / C + (C == 1 ? 5e3 : 18e3);
+    if (cost <= best) {
+      best = cost;
+      pl.C = C;
+      pl.threads = k == 1.0 ? 1024 : 512;
+    }
+  }
+  pl.most = (int)std::max(16.0, std::min(1024.0, 2e9 / best));
+  return pl;
+}
+
+static hp_status solve_laplace_clusters(hp_ctx* ctx, SolveProblem& pb, SolveResult& res, const ClusterPlan& pl) {
+  const int C = pl.C, most = pl.most;
+  const auto t0 = std::chrono::steady_clock::now();
+  const int nl = (int)pb.lats.size();
+  int Vmax = 0;
+  std::vector<SlotState> items;
+  res.qj.assign(nl, {});
+  res.qb.assign(nl, {});
+  for (int L = 0; L < nl; ++L) {
+    Vmax = std::max(Vmax, pb.lats[L].V);
+    const int dof = pb.lats[L].parts;
+    const size_t n = (size_t)(pb.s_max[L] - pb.first[L]) * dof;
+    res.qj[L].assign(n, make_double2(0.0, 0.0));
+    res.qb[L].assign(n, make_double2(0.0, 0.0));
+    for (int64_t m = pb.first[L]; m < pb.s_max[L]; ++m)
+      for (int k = 0; k < dof; ++k) {
+        SlotState S;
+        memset(&S, 0, sizeof(S));
+        S.status = SLOT_INIT;
+        S.lat = L;
+        S.m = (int)m;
+        S.a = k;
+        items.push_back(S);
+      }
+  }
+  const int n = (int)items.size();
+  // right-hand sides per launch: as many as are resident at once, up to 1 GB of vectors beyond that
+  const int resident = std::max(1, 2 * ctx->num_sms / C);
+  const int wave = (int)std::min<long long>(n, std::max<long long>(resident, (1LL << 30) / (32LL * Vmax)));
+  LArgs a;
+  memset(&a, 0, sizeof(a));
+  void* p = nullptr;
+  HP_TRY(hp_ws(ctx, "solve.lats", sizeof(LatGeom) * nl, &p));
+  HP_CUDA(cudaMemcpyAsync(p, pb.lats.data(), sizeof(LatGeom) * nl, cudaMemcpyHostToDevice, ctx->stream));
+  a.lats = (const LatGeom*)p;
+  HP_TRY(hp_ws(ctx, "solve.state", sizeof(SlotState) * (size_t)n, &p));
+  a.st = (SlotState*)p;
+  HP_CUDA(cudaMemcpyAsync(a.st, items.data(), sizeof(SlotState) * (size_t)n, cudaMemcpyHostToDevice, ctx->stream));
+  a.Vmax = Vmax;
+  a.nslots = wave;
+  a.tol2 = pb.tol * pb.tol;
+  a.maxiter = pb.opts.maxiter > 0 ? pb.opts.maxiter : 10000;
+  const char* names[4] = {"solve.lx", "solve.lr", "solve.lp", "solve.lq"};
+  double** v[4] = {&a.x, &a.r, &a.p, &a.q};
+  for (int k = 0; k < 4; ++k) {
+    HP_TRY(hp_ws(ctx, names[k], sizeof(double) * (size_t)wave * Vmax, &p));
+    *v[k] = (double*)p;
+  }
+  const int defl_k = pb.lats[0].defl_k;
+  if (defl_k) {
+    HP_TRY(hp_ws(ctx, "solve.defl_c", sizeof(double) * (size_t)n * defl_k, &p));
+    a.dc = (double*)p;
+    const int rows = 32768;   // grid limit of one dimension
+    for (int i0 = 0; i0 < n; i0 += rows) {
+      LArgs b = a;
+      b.st += i0;
+      b.dc += (size_t)i0 * defl_k;
+      ProfScope ps(ctx, "k_cg_defl");
+      k_cg_defl<256><<<dim3(defl_k, std::min(rows, n - i0)), 256, 0, ctx->stream>>>(b);
+    }
+    HP_LAUNCH_CHECK();
+  }
+  int* dev_slots = nullptr;
+  std::vector<int> ident;
+  if (pb.want_grad) {
+    HP_TRY(hp_ws(ctx, "solve.slots", sizeof(int) * (size_t)wave, &p));
+    dev_slots = (int*)p;
+    for (int i = 0; i < wave; ++i) ident.push_back(i);
+    HP_CUDA(cudaMemcpyAsync(dev_slots, ident.data(), sizeof(int) * ident.size(), cudaMemcpyHostToDevice, ctx->stream));
+  }
+  void (*kern)(LArgs, int, int, int) = pl.threads == 1024 ? k_cg_cluster<1024> : k_cg_cluster<512>;
+  for (int i0 = 0; i0 < n; i0 += wave) {
+    const int nw = std::min(wave, n - i0);
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(nw * C));
+    cfg.blockDim = dim3(pl.threads);
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = C;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    for (bool again = true; again;) {
+      {
+        ProfScope ps(ctx, "k_cg_cluster");
+        HP_CUDA(cudaLaunchKernelEx(&cfg, kern, a, i0, C, most));
+      }
+      again = false;
+      if (a.maxiter > most) {
+        HP_CUDA(cudaMemcpyAsync(items.data() + i0, a.st + i0, sizeof(SlotState) * (size_t)nw, cudaMemcpyDeviceToHost,
+                                ctx->stream));
+        HP_CUDA(cudaStreamSynchronize(ctx->stream));
+        for (int i = i0; i < i0 + nw; ++i) again = again || items[i].status == SLOT_RUN;
+      }
+    }
+    if (pb.want_grad) {
+      LArgs b = a;
+      b.st += i0;
+      for (int L = 0; L < nl; ++L) {
+        ProfScope ps(ctx, "k_lgrad");
+        k_lgrad<<<lblocks(ctx, pb.lats[L].V, 256), 256, 0, ctx->stream>>>(b, L, dev_slots, nw, pb.grad_dev[L], pb.lats[L].V);
+      }
+      HP_LAUNCH_CHECK();
+    }
+  }
+  HP_CUDA(cudaMemcpyAsync(items.data(), a.st, sizeof(SlotState) * (size_t)n, cudaMemcpyDeviceToHost, ctx->stream));
+  HP_CUDA(cudaStreamSynchronize(ctx->stream));
+  memset(&res.stats, 0, sizeof(res.stats));
+  res.stats.iterations_min = 0x7fffffff;
+  for (const SlotState& S : items) tally(S, pb.lats[S.lat].parts, pb, res);
+  if (res.stats.rhs_solved == 0) res.stats.iterations_min = 0;
+  res.stats.seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+  return HP_OK;
+}
+
 template <int SPL, bool MIXED>
 static hp_status run_blocked(hp_ctx* ctx, SolveProblem& pb, SolveResult& res) {
   BlockedSparseEngine<SPL, MIXED> e{ctx};
@@ -1284,6 +1585,17 @@ hp_status hp_solve_laplace(hp_ctx* ctx, SolveProblem& pb, SolveResult& res) {
     if (want <= 32) return run_blocked<1, false>(ctx, pb, res);
     if (want <= 64) return run_blocked<2, false>(ctx, pb, res);
     return run_blocked<4, false>(ctx, pb, res);
+  }
+  // the caller who fixes the slots, the chunk or the graph replay gets the slot engine
+  if (pb.opts.rhs_block <= 0 && pb.opts.check_every <= 0 && !pb.opts.use_graph) {
+    double n = 0.0, work = 0.0;
+    for (size_t L = 0; L < pb.lats.size(); ++L) {
+      const double k = (double)(pb.s_max[L] - pb.first[L]) * pb.lats[L].parts;
+      n += k;
+      work += k * pb.lats[L].V;
+    }
+    const ClusterPlan pl = cluster_plan(ctx, n, work / n);
+    if (pl.C && n <= 1e6) return solve_laplace_clusters(ctx, pb, res, pl);
   }
   LaplaceEngine e{ctx};
   return run_schedule(ctx, e, pb, res, 12, 0.0);

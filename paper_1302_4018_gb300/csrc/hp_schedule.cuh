@@ -13,6 +13,28 @@
 #include <chrono>
 #include <vector>
 
+// the result and statistics of one finished right-hand side (dof per probe)
+static inline void tally(const SlotState& S, int dof, const SolveProblem& pb, SolveResult& res) {
+  const int L = S.lat;
+  const size_t j = (size_t)(S.m - pb.first[L]) * dof + S.a;
+  res.qj[L][j] = S.q;
+  res.qb[L][j] = make_double2(S.gauss, S.gauss + S.radau * S.rnorm2);
+  res.stats.rhs_solved += 1;
+  res.stats.iterations_total += S.iters;
+  res.stats.iterations_max = std::max(res.stats.iterations_max, S.iters);
+  res.stats.iterations_min = std::min(res.stats.iterations_min, S.iters);
+  res.stats.reliable_updates += S.updates;
+  res.stats.sloppy_matvecs += S.sloppy_mv;
+  res.stats.fp64_matvecs += S.fp64_mv;
+  res.stats.group_updates += S.gupdates;
+  const double rel = S.bnorm2 > 0 ? std::sqrt(S.true_res2 / S.bnorm2) : 0.0;
+  res.stats.max_true_residual = std::max(res.stats.max_true_residual, rel);
+  if (S.status == SLOT_FAIL) {
+    res.stats.n_unconverged += 1;
+    res.unconverged = true;
+  }
+}
+
 template <class Engine>
 hp_status run_schedule(hp_ctx* ctx, Engine& eng, SolveProblem& pb, SolveResult& res, int dof_wilson, double delta) {
   auto t0 = std::chrono::steady_clock::now();
@@ -157,24 +179,7 @@ hp_status run_schedule(hp_ctx* ctx, Engine& eng, SolveProblem& pb, SolveResult& 
       HP_CUDA(cudaStreamSynchronize(ctx->stream));
       for (int sl : done) {
         SlotState& S = host[sl];
-        const int L = S.lat;
-        const int dof = pb.lats[L].op_kind == HP_OP_WILSON ? dof_wilson : pb.lats[L].parts;
-        res.qj[L][(size_t)(S.m - pb.first[L]) * dof + S.a] = S.q;
-        res.qb[L][(size_t)(S.m - pb.first[L]) * dof + S.a] = make_double2(S.gauss, S.gauss + S.radau * S.rnorm2);
-        res.stats.rhs_solved += 1;
-        res.stats.iterations_total += S.iters;
-        res.stats.iterations_max = std::max(res.stats.iterations_max, S.iters);
-        res.stats.iterations_min = std::min(res.stats.iterations_min, S.iters);
-        res.stats.reliable_updates += S.updates;
-        res.stats.sloppy_matvecs += S.sloppy_mv;
-        res.stats.fp64_matvecs += S.fp64_mv;
-        res.stats.group_updates += S.gupdates;
-        double rel = S.bnorm2 > 0 ? std::sqrt(S.true_res2 / S.bnorm2) : 0.0;
-        res.stats.max_true_residual = std::max(res.stats.max_true_residual, rel);
-        if (S.status == SLOT_FAIL) {
-          res.stats.n_unconverged += 1;
-          res.unconverged = true;
-        }
+        tally(S, pb.lats[S.lat].op_kind == HP_OP_WILSON ? dof_wilson : pb.lats[S.lat].parts, pb, res);
         S.status = SLOT_EMPTY;
       }
     }

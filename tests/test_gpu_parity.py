@@ -675,6 +675,50 @@ def test_wilson_apply_fp64_direct_and_in_place(ctx, hp, dims, nrhs, mf):
     assert np.abs(x.cpu().numpy() - ref).max() <= 200 * 2.3e-16 * np.abs(ref).max()
 
 
+# one right-hand side per cluster against the slot engine (rhs_block given): clusters of 1 to 8 blocks, ragged extents,
+# complex probes (two solves), a zero source, a mass field, an iteration limit, more iterations than one launch takes
+@pytest.mark.parametrize("dims,s,mass,mf,kind,maxiter", [
+    ((2, 2), 4, 0.3, 0, "hp", 0), ((7, 5, 3), 8, 0.3, 1, "z2", 0), ((6, 6, 6, 6), 40, 0.1, 0, "hp", 0),
+    ((16, 16, 8, 4), 3, 0.05, 1, "hp", 0), ((32, 30, 31), 16, 0.2, 0, "z2", 0), ((64, 64, 16), 20, 0.1, 1, "hp", 0),
+    ((12, 12, 12), 5, 1e-3, 0, "hp", 7), ((4099,), 2, 1e-5, 0, "z2", 0)])
+def test_laplacian_clusters_match_the_slot_engine(ctx, hp, dims, s, mass, mf, kind, maxiter):
+    mu = dev(np.abs(synth.mass_field(dims, 0.1, 9))) if mf else None
+    op = ctx.make_operator(hp.OP_LAPLACIAN, mass, mass_field=mu)
+    tol = 1e-12 if mass > 1e-4 else 1e-11
+    out = []
+    for block in (0, 8):
+        opts = ctx.make_opts("fp64", z0_seed=4, probe_kind=kind, rhs_block=block, maxiter=maxiter)
+        q = np.zeros(s, dtype=complex)
+        try:
+            T, q, st = ctx.trace_inv(op, dims, s, tol, opts, q)
+            out.append((q, st["n_unconverged"], st["rhs_solved"], st["iterations_max"]))
+            assert st["max_true_residual"] <= tol
+        except hp.HProbeError as e:
+            assert e.status == hp.HP_ENOCONV and maxiter == 7
+            out.append((q, -1, 0, 0))
+    (qa, ua, na, ia), (qb, ub, nb, ib) = out
+    assert ua == ub and na == nb and abs(ia - ib) <= max(2, ib // 10)
+    assert np.all(np.abs(qa - qb) <= 1e-9 * np.abs(qb))
+
+
+def test_laplacian_clusters_bounds_gradient_deflation(ctx, hp):
+    dims, s = (12, 10, 6), 6
+    V = int(np.prod(dims))
+    op = ctx.make_operator(hp.OP_LAPLACIAN, 0.2)
+    res = []
+    for block in (0, 4):
+        o = ctx.make_opts("fp64", z0_seed=4, rhs_block=block, probe_kind="z2")
+        T, lo, hi, _ = ctx.trace_inv_bounds(op, dims, s, 1e-9, o)
+        assert np.all(lo <= hi) and np.all(hi - lo <= 2e-9 * np.abs(hi))
+        g = np.zeros(V)
+        Tg, dm, _ = ctx.trace_inv_grad(op, dims, s, 1e-12, o, g)
+        W = np.ones((1, V)) / np.sqrt(V)   # the constant mode, eigenvalue = mass
+        Td, _, _ = ctx.trace_inv_deflated(op, dims, W, [0.2], s, 1e-12, o)
+        res.append((T, lo, hi, Tg, np.array([dm]), g, Td))
+    for a, b in zip(*res):
+        assert np.allclose(a, b, rtol=2e-9, atol=0)
+
+
 # ------------------------------------------------------------------ the comparison sequences (Section 5.2)
 @pytest.mark.parametrize("kind,dims,seed", [("natural", (8, 8, 8, 8), 0), ("natural", (2, 4, 8), 11),
                                             ("natural", (1024,), 3), ("z2", (4, 4, 4, 4), 12345),
