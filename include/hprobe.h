@@ -495,7 +495,7 @@ hp_status hp_sparse_probe_vectors(hp_ctx* ctx, int32_t n, const int32_t* paths, 
  * natural-order Hadamard / Z_2 sequences (1, 2; paths unused), each solved by
  * CG to a true relative residual tol computed in FP64 (complex probes as two
  * real solves).  The right-hand sides run in blocks of B = 32, 64 or 128
- * (opts->rhs_block rounded up; 0: 64) with the vectors stored [row][B].
+ * (opts->rhs_block rounded up; 0: by the number of right-hand sides) with the vectors stored [row][B].
  * opts->precision: HP_PREC_FP64, or HP_PREC_MIXED_FP32 = FP32 iteration with
  * FP64 reliable updates (a true residual whenever ||r|| fell by opts->delta,
  * default 1e-5, since the last one).  q_inout, trace_prefix, stats as

@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "hp_internal.h"
 
@@ -561,20 +562,21 @@ struct LaplaceEngine {
 
 // ------------------------------------------------------------ blocked sparse CG
 // A general sparse matrix runs all B = 32 SPL slots as one block of vectors laid out
-// [row][slot] (lane l of a warp owns slots l, l + 32, ...).  One warp per row reads the row's
-// CSR entries once for every slot and gathers B contiguous values per entry (256 SPL bytes,
-// whole sectors), where one slot per block row would re-read the matrix for every slot and
-// gather single words.  Reductions: each block leaves per-slot partial sums, the last block
-// to finish adds them in a fixed order and takes the scalar CG steps of every slot.
+// [row][slot] (lane l of a warp owns the slots l SPL .. l SPL + SPL - 1).  One warp per row reads the row's
+// CSR entries once for every slot and gathers B contiguous values per entry (whole sectors), where one slot
+// per block row would re-read the matrix for every slot and gather single words.  Reductions: each block
+// leaves its sum per slot, the last block of 32 adds theirs, the last of those adds the groups' sums in
+// a fixed order and takes the scalar CG steps of every slot.
 struct BArgs {
   const LatGeom* lat;
   SlotState* st;
   double *x, *r, *p, *q;   // [n][B]
-  double* part;            // [B][nblk]
-  unsigned int* cnt;       // one counter per reducing kernel
+  double* part;            // [blocks][B]
+  double* gpart;           // [groups of 32 blocks][B]
+  unsigned int* cnt;       // per reducing kernel: one counter, then one per group
+  int ngroups_max;
   int nblk;               // blocks of the matrix-vector kernels
   int nstream;            // blocks of the streaming kernels
-  int pstride;            // row stride of part: max(nblk, nstream)
   double tol2;
   int maxiter;
   // mixed precision: r, p, q and the correction xl in FP32, x = xh + xl with xh in FP64
@@ -596,72 +598,91 @@ __device__ __forceinline__ bool bk_on(const SlotState* S, int kind) {
   }
 }
 
-template <int SPL>
-__device__ __forceinline__ void bk_finish(const BArgs& a, const LatGeom& g, int kind, const double (&acc)[SPL]) {
-  constexpr int B = 32 * SPL, NW = BT / 32;
-  __shared__ double sh[NW][B];
-  __shared__ double tot_sh[B];
+// N neighbouring slots of a row, moved in 16-byte pieces
+template <typename T, int N>
+struct alignas(sizeof(T) * N > 16 ? 16 : sizeof(T) * N) Pack {
+  T v[N];
+};
+
+// t: the block's sum of slot threadIdx.x (threads < B).  The FP64 additions of one block over all partial sums (64 slots
+// x 1216 blocks: 2400 warp instructions at 16 cycles, 20 us at the end of every launch) run in groups side by side.
+template <int B>
+__device__ __forceinline__ void bk_finish(const BArgs& a, const LatGeom& g, int kind, double t) {
   __shared__ int am_last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < SPL; ++k) sh[warp][lane + 32 * k] = acc[k];
-  __syncthreads();
-  if (threadIdx.x < B) {
-    double t = 0.0;
-    for (int w = 0; w < NW; ++w) t += sh[w][threadIdx.x];
-    a.part[(size_t)threadIdx.x * a.pstride + blockIdx.x] = t;
-  }
+  const int nb = gridDim.x, grp = blockIdx.x >> 5, ng = (nb + 31) >> 5, members = min(32, nb - 32 * grp);
+  unsigned int* cnt = a.cnt + kind * (1 + a.ngroups_max);
+  if (threadIdx.x < B) a.part[(size_t)blockIdx.x * B + threadIdx.x] = t;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) am_last = atomicAdd(a.cnt + kind, 1u) == (unsigned)gridDim.x - 1u;
+  if (threadIdx.x == 0) am_last = atomicAdd(cnt + 1 + grp, 1u) == (unsigned)members - 1u;
   __syncthreads();
   if (!am_last) return;
   __threadfence();
-  // warp w adds up the partials of slots w, w + NW, ...: lanes run over the blocks (coalesced
-  // loads, four independent sums each), then a shuffle tree; the order is fixed
-  const int nb = gridDim.x;
-  for (int s = warp; s < B; s += NW) {
-    const double* ps = a.part + (size_t)s * a.pstride;
-    double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;
-    int j = lane;
-    for (; j + 96 < nb; j += 128) {
-      t0 += __ldcg(ps + j);
-      t1 += __ldcg(ps + j + 32);
-      t2 += __ldcg(ps + j + 64);
-      t3 += __ldcg(ps + j + 96);
-    }
-    for (; j < nb; j += 32) t0 += __ldcg(ps + j);
-    double t = (t0 + t1) + (t2 + t3);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) tot_sh[s] = t;
-  }
-  __syncthreads();
   if (threadIdx.x < B) {
-    const double tot = tot_sh[threadIdx.x];
+    const double* ps = a.part + (size_t)32 * grp * B + threadIdx.x;
+    t = 0.0;
+#pragma unroll 8
+    for (int k = 0; k < members; ++k) t += __ldcg(ps + (size_t)k * B);
+    a.gpart[(size_t)grp * B + threadIdx.x] = t;
+  }
+  if (threadIdx.x == 0) cnt[1 + grp] = 0;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) am_last = atomicAdd(cnt, 1u) == (unsigned)ng - 1u;
+  __syncthreads();
+  if (!am_last) return;
+  __threadfence();
+  if (threadIdx.x < B) {
+    double tot = 0.0;
+#pragma unroll 8
+    for (int k = 0; k < ng; ++k) tot += __ldcg(a.gpart + (size_t)k * B + threadIdx.x);
     SlotState* S = a.st + threadIdx.x;
     if (bk_on(S, kind)) {
       switch (kind) {
         case BK_INIT: cg_after_init(S, g, tot); break;
         case BK_AP: cg_after_ap(S, tot); break;
         case BK_XR: cg_after_xr(S, g, tot, a.tol2, a.maxiter, a.delta2); break;
-        case BK_TRUE: cg_after_true(S, tot, a.tol2, a.xl != nullptr); break;
         default: S->q = make_double2(tot, 0.0); break;
       }
     }
   }
-  if (threadIdx.x == 0) a.cnt[kind] = 0;
+  if (threadIdx.x == 0) *cnt = 0;
+}
+
+// the block's sum of slot threadIdx.x (threads < 32 SPL) from the lanes' sums of the slots they own
+template <int SPL, typename T>
+__device__ __forceinline__ double bk_sum_lanes(const T (&acc)[SPL]) {
+  constexpr int B = 32 * SPL, NW = BT / 32;
+  __shared__ T sh[NW][B];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < SPL; ++k) sh[warp][lane * SPL + k] = acc[k];
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < B)
+#pragma unroll
+    for (int w = 0; w < NW; ++w) t += (double)sh[w][threadIdx.x];
+  return t;
+}
+// the same for the streaming kernels, where thread t holds the sums of the VW slots from (t % (B / VW)) VW on
+template <int B, int VW, typename T>
+__device__ __forceinline__ double bk_sum_cols(const T (&acc)[VW]) {
+  constexpr int TPR = B / VW;
+  __shared__ T sh[BT / TPR][B];
+#pragma unroll
+  for (int k = 0; k < VW; ++k) sh[threadIdx.x / TPR][(threadIdx.x % TPR) * VW + k] = acc[k];
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < B)
+#pragma unroll
+    for (int w = 0; w < BT / TPR; ++w) t += (double)sh[w][threadIdx.x];
+  return t;
 }
 
 #define BK_ROWS(i) for (int i = blockIdx.x * (BT / 32) + (threadIdx.x >> 5); i < g.V; i += gridDim.x * (BT / 32))
-// rows i0 + u tw, u < BR, per warp and step: a streaming kernel issues all their loads first
-constexpr int BR = 4;
-#define BK_ROW_BATCHES(i0, tw)                            \
-  const int tw = gridDim.x * (BT / 32);                   \
-  for (int i0 = blockIdx.x * (BT / 32) + (threadIdx.x >> 5); i0 < g.V; i0 += BR * tw)
 
-// x = 0, r = p = b for the slots being filled; ||b||^2
-template <int SPL>
+// x = 0, r = p = b for the slots being filled; ||b||^2  (MIXED: r, p and the correction in FP32)
+template <int SPL, bool MIXED>
 __global__ void __launch_bounds__(BT) k_bcg_init(BArgs a) {
   constexpr int B = 32 * SPL;
   const LatGeom g = *a.lat;
@@ -671,7 +692,7 @@ __global__ void __launch_bounds__(BT) k_bcg_init(BArgs a) {
   double acc[SPL];
 #pragma unroll
   for (int k = 0; k < SPL; ++k) {
-    const SlotState* S = a.st + lane + 32 * k;
+    const SlotState* S = a.st + lane * SPL + k;
     on[k] = bk_on(S, BK_INIT);
     m[k] = S->m;
     pa[k] = S->a;
@@ -681,203 +702,216 @@ __global__ void __launch_bounds__(BT) k_bcg_init(BArgs a) {
 #pragma unroll
     for (int k = 0; k < SPL; ++k) {
       if (!on[k]) continue;
-      const size_t o = (size_t)i * B + lane + 32 * k;
+      const size_t o = (size_t)i * B + lane * SPL + k;
       const double b = lap_source(g, i, m[k], pa[k]);
       a.x[o] = 0.0;
-      a.r[o] = b;
-      a.p[o] = b;
+      if (MIXED) {
+        a.xl[o] = 0.0f;
+        a.rf[o] = (float)b;
+        a.pf[o] = (float)b;
+      } else {
+        a.r[o] = b;
+        a.p[o] = b;
+      }
       acc[k] += b * b;
     }
   }
-  bk_finish<SPL>(a, g, BK_INIT, acc);
+  bk_finish<B>(a, g, BK_INIT, bk_sum_lanes<SPL>(acc));
 }
 
-// (A v)[i][slot] for the rows r0 .. r1-1 of one warp, handed to flush(i, value, own) row by row
-// in order, with own = own_src[i][slot] (own_src may be NULL).  The rows'
-// CSR entries are contiguous: the warp loads them 32 at a time (one entry per lane, coalesced;
-// the next 32 are requested before the current ones are used), broadcasts each entry, and
-// issues U gathers of B contiguous values before it adds them.  Each warp walks a long chain of
-// dependent loads, so every load that can be issued early is.
-template <int SPL, typename T, int U = 8, class Flush>
-__device__ __forceinline__ void bk_spmv_rows(const LatGeom& g, const T* __restrict__ val, const T* __restrict__ v,
-                                             const T* __restrict__ own_src, int r0, int r1, int lane,
-                                             const bool (&on)[SPL], Flush&& flush) {
-  constexpr int B = 32 * SPL;
+// q = A p, (p, q): in FP64, or (MIXED) in FP32 with the block sums in FP64.
+// A warp walks rows gw, gw + tw, ...: the row pointers two rows ahead and the entries one row ahead are requested before the
+// gathers of the current row, so a row costs the warp one memory latency (its gathers, eight at a time in flight), and
+// the resident warps cover it.  A walk over contiguous rows of one entry stream, flushing rows as they ended, spent
+// 153 us where this takes 87 (64^3 grid renumbered, B = 64, FP32; 134 MB of p and q plus 470 MB of gathers from L2).
+template <int SPL, bool MIXED>
+__global__ void __launch_bounds__(BT, SPL == 4 ? (MIXED ? 4 : 2) : 4) k_bcg_ap(BArgs a) {
+  typedef typename std::conditional<MIXED, float, double>::type T;
+  typedef Pack<T, SPL> P;
+  constexpr int B = 32 * SPL, U = sizeof(P) >= 16 ? 4 : 8;
   constexpr unsigned FULL = 0xffffffffu;
-  if (r0 >= r1) return;
-  int i = r0, rbase = r0;
-  int rend_l = (rbase + lane < r1) ? __ldg(g.csr_rp + rbase + lane + 1) : 0x7fffffff;
-  int row_end = __shfl_sync(FULL, rend_l, 0);
-  T acc[SPL], own[SPL];
+  const LatGeom& g = *a.lat;   // by reference: a copy of the struct costs 20 registers
+  const int V = g.V;
+  const int *__restrict__ rp = g.csr_rp, *__restrict__ ci = g.csr_ci;
+  const int lane = threadIdx.x & 31;
+  const T* __restrict__ val = MIXED ? (const T*)a.val32 : (const T*)g.csr_val;
+  const T* __restrict__ v = MIXED ? (const T*)a.pf : (const T*)a.p;
+  T* __restrict__ q = MIXED ? (T*)a.qf : (T*)a.q;
+  bool any = false;   // lanes whose slots all rest neither load nor store (an idle slot's q may be overwritten)
+  T dot[SPL];
 #pragma unroll
-  for (int k = 0; k < SPL; ++k) acc[k] = T(0);
-  auto advance = [&](int e) {   // flush every row that ends at entry e (empty rows included)
-    while (i < r1 && row_end == e) {
-#pragma unroll
-      for (int k = 0; k < SPL; ++k) own[k] = (own_src && on[k]) ? own_src[(size_t)i * B + lane + 32 * k] : T(0);
-      flush(i, acc, own);
-#pragma unroll
-      for (int k = 0; k < SPL; ++k) acc[k] = T(0);
-      ++i;
-      if (i - rbase == 32) {
-        rbase = i;
-        rend_l = (rbase + lane < r1) ? __ldg(g.csr_rp + rbase + lane + 1) : 0x7fffffff;
-      }
-      if (i < r1) row_end = __shfl_sync(FULL, rend_l, i - rbase);
+  for (int k = 0; k < SPL; ++k) {
+    any |= bk_on(a.st + lane * SPL + k, BK_AP);
+    dot[k] = T(0);
+  }
+  const int tw = gridDim.x * (BT / 32);
+  int i = blockIdx.x * (BT / 32) + (threadIdx.x >> 5);
+  int b = 0, e = 0, b2 = 0, e2 = 0, c = 0;
+  T w = T(0);
+  if (i < V) {
+    b = __ldg(rp + i);
+    e = __ldg(rp + i + 1);
+    if (i + tw < V) {
+      b2 = __ldg(rp + i + tw);
+      e2 = __ldg(rp + i + tw + 1);
     }
-  };
-  const int e_beg = __ldg(g.csr_rp + r0), e_fin = __ldg(g.csr_rp + r1);
-  advance(e_beg);
-  int c_n = e_beg + lane < e_fin ? __ldg(g.csr_ci + e_beg + lane) : 0;
-  T w_n = e_beg + lane < e_fin ? __ldg(val + e_beg + lane) : T(0);
-  for (int e0 = e_beg; e0 < e_fin; e0 += 32) {
-    const int nb = min(32, e_fin - e0);
-    const int c_l = c_n;
-    const T w_l = w_n;
-    const int en = e0 + 32 + lane;   // the next 32 entries, requested now
-    c_n = en < e_fin ? __ldg(g.csr_ci + en) : 0;
-    w_n = en < e_fin ? __ldg(val + en) : T(0);
-    for (int j0 = 0; j0 < nb; j0 += U) {
-      T gv[U][SPL];
+    if (b + lane < e) {
+      c = __ldg(ci + b + lane);
+      w = __ldg(val + b + lane);
+    }
+  }
+  for (; i < V; i += tw) {
+    int b3 = 0, e3 = 0, c2 = 0;
+    T w2 = T(0);
+    if (b2 + lane < e2) {
+      c2 = __ldg(ci + b2 + lane);
+      w2 = __ldg(val + b2 + lane);
+    }
+    if ((long long)i + 2LL * tw < V) {
+      b3 = __ldg(rp + i + 2 * tw);
+      e3 = __ldg(rp + i + 2 * tw + 1);
+    }
+    P own, acc;
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int c = __shfl_sync(FULL, c_l, j0 + u);   // lanes past nb hold row 0: in bounds, unused
-        const T* vj = v + (size_t)c * B + lane;
-#pragma unroll
-        for (int k = 0; k < SPL; ++k) gv[u][k] = (on[k] && j0 + u < nb) ? vj[32 * k] : T(0);
+    for (int k = 0; k < SPL; ++k) own.v[k] = acc.v[k] = T(0);
+    if (any) own = *reinterpret_cast<const P*>(v + (size_t)i * B + lane * SPL);
+    for (int e0 = b; e0 < e; e0 += 32) {
+      const int n = min(32, e - e0);
+      if (e0 != b) {   // a row of more than 32 entries
+        c = lane < n ? __ldg(ci + e0 + lane) : 0;
+        w = lane < n ? __ldg(val + e0 + lane) : T(0);
       }
+      for (int j0 = 0; j0 < n; j0 += U) {
+        P gv[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (j0 + u < nb) {
-          const T w = __shfl_sync(FULL, w_l, j0 + u);
+        for (int u = 0; u < U; ++u) {
+          const int cj = __shfl_sync(FULL, c, j0 + u);
 #pragma unroll
-          for (int k = 0; k < SPL; ++k) acc[k] += w * gv[u][k];
-          advance(e0 + j0 + u + 1);
+          for (int k = 0; k < SPL; ++k) gv[u].v[k] = T(0);
+          if (any && j0 + u < n) gv[u] = *reinterpret_cast<const P*>(v + (size_t)cj * B + lane * SPL);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const T wj = __shfl_sync(FULL, w, j0 + u);   // lanes past the row hold 0
+#pragma unroll
+          for (int k = 0; k < SPL; ++k) acc.v[k] = fma(j0 + u < n ? wj : T(0), gv[u].v[k], acc.v[k]);
         }
       }
     }
-  }
-}
-
-// the contiguous rows of warp number gw of tw warps
-__device__ __forceinline__ void bk_warp_rows(int n, int& r0, int& r1) {
-  const int tw = gridDim.x * (BT / 32), gw = blockIdx.x * (BT / 32) + (threadIdx.x >> 5);
-  const int chunk = (n + tw - 1) / tw;
-  r0 = min(n, gw * chunk);
-  r1 = min(n, r0 + chunk);
-}
-
-// q = A p ; (p, q)
-template <int SPL>
-__global__ void __launch_bounds__(BT, SPL == 1 ? 4 : (SPL == 2 ? 3 : 2)) k_bcg_ap(BArgs a) {
-  constexpr int B = 32 * SPL;
-  const LatGeom g = *a.lat;
-  const int lane = threadIdx.x & 31;
-  bool on[SPL];
-  double acc[SPL];
+    if (any) {
+      *reinterpret_cast<P*>(q + (size_t)i * B + lane * SPL) = acc;
 #pragma unroll
-  for (int k = 0; k < SPL; ++k) {
-    on[k] = bk_on(a.st + lane + 32 * k, BK_AP);
-    acc[k] = 0.0;
-  }
-  int r0, r1;
-  bk_warp_rows(g.V, r0, r1);
-  bk_spmv_rows<SPL, double>(g, g.csr_val, a.p, a.p, r0, r1, lane, on, [&](int i, const double (&qv)[SPL], const double (&pv)[SPL]) {
-#pragma unroll
-    for (int k = 0; k < SPL; ++k) {
-      if (!on[k]) continue;
-      a.q[(size_t)i * B + lane + 32 * k] = qv[k];
-      acc[k] += pv[k] * qv[k];
+      for (int k = 0; k < SPL; ++k) dot[k] = fma(own.v[k], acc.v[k], dot[k]);
     }
-  });
-  bk_finish<SPL>(a, g, BK_AP, acc);
+    b = b2, e = e2, b2 = b3, e2 = e3, c = c2, w = w2;
+  }
+  bk_finish<B>(a, g, BK_AP, bk_sum_lanes<SPL>(dot));
 }
 
-// x += alpha p ; r -= alpha q ; (r, r)
-template <int SPL>
-__global__ void __launch_bounds__(BT) k_bcg_xr(BArgs a) {
-  constexpr int B = 32 * SPL;
-  const LatGeom g = *a.lat;
-  const int lane = threadIdx.x & 31;
-  bool on[SPL];
-  double al[SPL], acc[SPL];
+// The streaming kernels: a thread owns VW neighbouring slots (16 bytes) of every (blocks BT / TPR)-th row and takes BR rows
+// at a time, all loads first.  Slots at rest keep their values: a thread without a running slot skips its loads, the
+// others write back what they read.
+constexpr int BR = 2;
+#define BK_STREAM(B, VW)                                                                                     \
+  constexpr int TPR = (B) / (VW);                                                                            \
+  const int slot0 = (int)(threadIdx.x % TPR) * (VW);                                                         \
+  const int tw = (int)gridDim.x * (BT / TPR), row0 = (int)blockIdx.x * (BT / TPR) + (int)threadIdx.x / TPR;
+
+// x += alpha p ; r -= alpha q ; (r, r)   (MIXED: the correction xl, r, p, q and the lane sums in FP32)
+template <int SPL, bool MIXED>
+__global__ void __launch_bounds__(BT, 4) k_bcg_xr(BArgs a) {
+  typedef typename std::conditional<MIXED, float, double>::type T;
+  constexpr int B = 32 * SPL, VW = 16 / sizeof(T);
+  typedef Pack<T, VW> P;
+  const LatGeom& g = *a.lat;
+  const int V = g.V;
+  BK_STREAM(B, VW)
+  bool on[VW], any = false;
+  T al[VW], acc[VW];
 #pragma unroll
-  for (int k = 0; k < SPL; ++k) {
-    const SlotState* S = a.st + lane + 32 * k;
+  for (int k = 0; k < VW; ++k) {
+    const SlotState* S = a.st + slot0 + k;
     on[k] = bk_on(S, BK_XR);
-    al[k] = S->alpha.x;
-    acc[k] = 0.0;
+    any |= on[k];
+    al[k] = (T)S->alpha.x;
+    acc[k] = T(0);
   }
-  double* __restrict__ x = a.x;
-  double* __restrict__ r = a.r;
-  const double* __restrict__ p = a.p;
-  const double* __restrict__ q = a.q;
-  BK_ROW_BATCHES(i0, tw) {   // loads of BR rows first, then the updates: BR x 4 SPL loads in flight
-    double xv[BR][SPL], pv[BR][SPL], qv[BR][SPL], rv[BR][SPL];
+  T* __restrict__ x = MIXED ? (T*)a.xl : (T*)a.x;
+  T* __restrict__ r = MIXED ? (T*)a.rf : (T*)a.r;
+  const T* __restrict__ p = MIXED ? (const T*)a.pf : (const T*)a.p;
+  const T* __restrict__ q = MIXED ? (const T*)a.qf : (const T*)a.q;
+  if (any)
+    for (long long i0 = row0; i0 < V; i0 += (long long)BR * tw) {
+      P xv[BR], pv[BR], qv[BR], rv[BR];
 #pragma unroll
-    for (int u = 0; u < BR; ++u)
-#pragma unroll
-      for (int k = 0; k < SPL; ++k) {
-        const int i = i0 + u * tw;
-        if (i >= g.V || !on[k]) continue;
-        const size_t o = (size_t)i * B + lane + 32 * k;
-        xv[u][k] = x[o];
-        pv[u][k] = p[o];
-        qv[u][k] = q[o];
-        rv[u][k] = r[o];
+      for (int u = 0; u < BR; ++u) {
+        const long long i = i0 + (long long)u * tw;
+        if (i >= V) continue;
+        const size_t o = (size_t)i * B + slot0;
+        xv[u] = *reinterpret_cast<const P*>(x + o);
+        pv[u] = *reinterpret_cast<const P*>(p + o);
+        qv[u] = *reinterpret_cast<const P*>(q + o);
+        rv[u] = *reinterpret_cast<const P*>(r + o);
       }
 #pragma unroll
-    for (int u = 0; u < BR; ++u)
+      for (int u = 0; u < BR; ++u) {
+        const long long i = i0 + (long long)u * tw;
+        if (i >= V) continue;
+        const size_t o = (size_t)i * B + slot0;
 #pragma unroll
-      for (int k = 0; k < SPL; ++k) {
-        const int i = i0 + u * tw;
-        if (i >= g.V || !on[k]) continue;
-        const size_t o = (size_t)i * B + lane + 32 * k;
-        x[o] = xv[u][k] + al[k] * pv[u][k];
-        const double rn = rv[u][k] - al[k] * qv[u][k];
-        r[o] = rn;
-        acc[k] += rn * rn;
+        for (int k = 0; k < VW; ++k) {
+          const T rn = fma(-al[k], qv[u].v[k], rv[u].v[k]), xn = fma(al[k], pv[u].v[k], xv[u].v[k]);
+          if (on[k]) {
+            xv[u].v[k] = xn;
+            rv[u].v[k] = rn;
+            acc[k] = fma(rn, rn, acc[k]);
+          }
+        }
+        *reinterpret_cast<P*>(x + o) = xv[u];
+        *reinterpret_cast<P*>(r + o) = rv[u];
       }
-  }
-  bk_finish<SPL>(a, g, BK_XR, acc);
+    }
+  bk_finish<B>(a, g, BK_XR, bk_sum_cols<B, VW>(acc));
 }
 
 // p = r + beta p
-template <int SPL>
-__global__ void __launch_bounds__(BT) k_bcg_p(BArgs a) {
-  constexpr int B = 32 * SPL;
-  const LatGeom g = *a.lat;
-  const int lane = threadIdx.x & 31;
-  bool on[SPL];
-  double be[SPL];
+template <int SPL, bool MIXED>
+__global__ void __launch_bounds__(BT, 4) k_bcg_p(BArgs a) {
+  typedef typename std::conditional<MIXED, float, double>::type T;
+  constexpr int B = 32 * SPL, VW = 16 / sizeof(T);
+  typedef Pack<T, VW> P;
+  const int V = a.lat->V;
+  BK_STREAM(B, VW)
+  bool on[VW], any = false;
+  T be[VW];
 #pragma unroll
-  for (int k = 0; k < SPL; ++k) {
-    const SlotState* S = a.st + lane + 32 * k;
+  for (int k = 0; k < VW; ++k) {
+    const SlotState* S = a.st + slot0 + k;
     on[k] = S->status == SLOT_RUN;
-    be[k] = S->restart ? 0.0 : S->beta.x;
+    any |= on[k];
+    be[k] = S->restart ? T(0) : (T)S->beta.x;
   }
-  double* __restrict__ p = a.p;
-  const double* __restrict__ r = a.r;
-  BK_ROW_BATCHES(i0, tw) {
-    double pv[BR][SPL], rv[BR][SPL];
+  if (!any) return;
+  T* __restrict__ p = MIXED ? (T*)a.pf : (T*)a.p;
+  const T* __restrict__ r = MIXED ? (const T*)a.rf : (const T*)a.r;
+  for (long long i0 = row0; i0 < V; i0 += (long long)BR * tw) {
+    P pv[BR], rv[BR];
 #pragma unroll
-    for (int u = 0; u < BR; ++u)
+    for (int u = 0; u < BR; ++u) {
+      const long long i = i0 + (long long)u * tw;
+      if (i >= V) continue;
+      pv[u] = *reinterpret_cast<const P*>(p + (size_t)i * B + slot0);
+      rv[u] = *reinterpret_cast<const P*>(r + (size_t)i * B + slot0);
+    }
 #pragma unroll
-      for (int k = 0; k < SPL; ++k) {
-        const int i = i0 + u * tw;
-        if (i >= g.V || !on[k]) continue;
-        const size_t o = (size_t)i * B + lane + 32 * k;
-        pv[u][k] = p[o];
-        rv[u][k] = r[o];
-      }
+    for (int u = 0; u < BR; ++u) {
+      const long long i = i0 + (long long)u * tw;
+      if (i >= V) continue;
 #pragma unroll
-    for (int u = 0; u < BR; ++u)
-#pragma unroll
-      for (int k = 0; k < SPL; ++k) {
-        const int i = i0 + u * tw;
-        if (i >= g.V || !on[k]) continue;
-        p[(size_t)i * B + lane + 32 * k] = rv[u][k] + be[k] * pv[u][k];
-      }
+      for (int k = 0; k < VW; ++k)
+        if (on[k]) pv[u].v[k] = fma(be[k], pv[u].v[k], rv[u].v[k]);
+      *reinterpret_cast<P*>(p + (size_t)i * B + slot0) = pv[u];
+    }
   }
 }
 
@@ -892,7 +926,7 @@ __global__ void __launch_bounds__(BT) k_bcg_quad(BArgs a) {
   double acc[SPL];
 #pragma unroll
   for (int k = 0; k < SPL; ++k) {
-    const SlotState* S = a.st + lane + 32 * k;
+    const SlotState* S = a.st + lane * SPL + k;
     on[k] = bk_on(S, BK_QUAD);
     m[k] = S->m;
     pa[k] = S->a;
@@ -901,132 +935,14 @@ __global__ void __launch_bounds__(BT) k_bcg_quad(BArgs a) {
   BK_ROWS(i) {
 #pragma unroll
     for (int k = 0; k < SPL; ++k)
-      if (on[k]) acc[k] += lap_source(g, i, m[k], pa[k]) * a.x[(size_t)i * B + lane + 32 * k];
+      if (on[k]) acc[k] += lap_source(g, i, m[k], pa[k]) * a.x[(size_t)i * B + lane * SPL + k];
   }
-  bk_finish<SPL>(a, g, BK_QUAD, acc);
+  bk_finish<B>(a, g, BK_QUAD, bk_sum_lanes<SPL>(acc));
 }
 
-// ---- mixed precision (FP32 iteration, FP64 reliable updates): the matrix-vector product,
-// the recurrences and the per-lane dot products in FP32; ||b||^2, the block sums and the true
-// residual b - A (xh + xl) in FP64.  A reliable update folds xl into xh, recomputes r in FP64
-// and keeps p.
-
-// xh = 0, xl = 0, r = p = b
-template <int SPL>
-__global__ void __launch_bounds__(BT) k_bcm_init(BArgs a) {
-  constexpr int B = 32 * SPL;
-  const LatGeom g = *a.lat;
-  const int lane = threadIdx.x & 31;
-  bool on[SPL];
-  int m[SPL], pa[SPL];
-  double acc[SPL];
-#pragma unroll
-  for (int k = 0; k < SPL; ++k) {
-    const SlotState* S = a.st + lane + 32 * k;
-    on[k] = bk_on(S, BK_INIT);
-    m[k] = S->m;
-    pa[k] = S->a;
-    acc[k] = 0.0;
-  }
-  BK_ROWS(i) {
-#pragma unroll
-    for (int k = 0; k < SPL; ++k) {
-      if (!on[k]) continue;
-      const size_t o = (size_t)i * B + lane + 32 * k;
-      const double b = lap_source(g, i, m[k], pa[k]);
-      a.x[o] = 0.0;
-      a.xl[o] = 0.0f;
-      a.rf[o] = (float)b;
-      a.pf[o] = (float)b;
-      acc[k] += b * b;
-    }
-  }
-  bk_finish<SPL>(a, g, BK_INIT, acc);
-}
-
-// q = A p, (p, q) in FP32
-template <int SPL>
-__global__ void __launch_bounds__(BT, SPL <= 2 ? 4 : 2) k_bcm_ap(BArgs a) {
-  constexpr int B = 32 * SPL;
-  const LatGeom g = *a.lat;
-  const int lane = threadIdx.x & 31;
-  bool on[SPL];
-  float accf[SPL];
-#pragma unroll
-  for (int k = 0; k < SPL; ++k) {
-    on[k] = bk_on(a.st + lane + 32 * k, BK_AP);
-    accf[k] = 0.0f;
-  }
-  int r0, r1;
-  bk_warp_rows(g.V, r0, r1);
-  bk_spmv_rows<SPL, float, 16>(g, a.val32, a.pf, a.pf, r0, r1, lane, on,
-                           [&](int i, const float (&qv)[SPL], const float (&pv)[SPL]) {
-#pragma unroll
-                             for (int k = 0; k < SPL; ++k) {
-                               if (!on[k]) continue;
-                               a.qf[(size_t)i * B + lane + 32 * k] = qv[k];
-                               accf[k] = fmaf(pv[k], qv[k], accf[k]);
-                             }
-                           });
-  double acc[SPL];
-#pragma unroll
-  for (int k = 0; k < SPL; ++k) acc[k] = accf[k];
-  bk_finish<SPL>(a, g, BK_AP, acc);
-}
-
-// xl += alpha p, r -= alpha q, (r, r) in FP32
-template <int SPL>
-__global__ void __launch_bounds__(BT) k_bcm_xr(BArgs a) {
-  constexpr int B = 32 * SPL;
-  const LatGeom g = *a.lat;
-  const int lane = threadIdx.x & 31;
-  bool on[SPL];
-  float al[SPL], accf[SPL];
-#pragma unroll
-  for (int k = 0; k < SPL; ++k) {
-    const SlotState* S = a.st + lane + 32 * k;
-    on[k] = bk_on(S, BK_XR);
-    al[k] = (float)S->alpha.x;
-    accf[k] = 0.0f;
-  }
-  float* __restrict__ xl = a.xl;
-  float* __restrict__ rf = a.rf;
-  const float* __restrict__ pf = a.pf;
-  const float* __restrict__ qf = a.qf;
-  BK_ROW_BATCHES(i0, tw) {
-    float xv[BR][SPL], pv[BR][SPL], qv[BR][SPL], rv[BR][SPL];
-#pragma unroll
-    for (int u = 0; u < BR; ++u)
-#pragma unroll
-      for (int k = 0; k < SPL; ++k) {
-        const int i = i0 + u * tw;
-        if (i >= g.V || !on[k]) continue;
-        const size_t o = (size_t)i * B + lane + 32 * k;
-        xv[u][k] = xl[o];
-        pv[u][k] = pf[o];
-        qv[u][k] = qf[o];
-        rv[u][k] = rf[o];
-      }
-#pragma unroll
-    for (int u = 0; u < BR; ++u)
-#pragma unroll
-      for (int k = 0; k < SPL; ++k) {
-        const int i = i0 + u * tw;
-        if (i >= g.V || !on[k]) continue;
-        const size_t o = (size_t)i * B + lane + 32 * k;
-        xl[o] = fmaf(al[k], pv[u][k], xv[u][k]);
-        const float rn = fmaf(-al[k], qv[u][k], rv[u][k]);
-        rf[o] = rn;
-        accf[k] = fmaf(rn, rn, accf[k]);
-      }
-  }
-  double acc[SPL];
-#pragma unroll
-  for (int k = 0; k < SPL; ++k) acc[k] = accf[k];
-  bk_finish<SPL>(a, g, BK_XR, acc);
-}
-
-// reliable update, first half: xh += xl, xl = 0 for the slots that asked for a true residual
+// reliable update, first half (mixed precision: the matrix-vector product, the recurrences and the per-lane dot products
+// run in FP32; ||b||^2, the block sums and the true residual b - A (xh + xl) in FP64): xh += xl, xl = 0 for the
+// slots that asked for a true residual, which then recomputes r in FP64 and keeps p
 template <int SPL>
 __global__ void __launch_bounds__(BT) k_bcm_fold(BArgs a) {
   constexpr int B = 32 * SPL;
@@ -1036,7 +952,7 @@ __global__ void __launch_bounds__(BT) k_bcm_fold(BArgs a) {
   bool any = false;
 #pragma unroll
   for (int k = 0; k < SPL; ++k) {
-    on[k] = bk_on(a.st + lane + 32 * k, BK_TRUE);
+    on[k] = bk_on(a.st + lane * SPL + k, BK_TRUE);
     any |= on[k];
   }
   if (!__syncthreads_or(any)) return;
@@ -1044,84 +960,86 @@ __global__ void __launch_bounds__(BT) k_bcm_fold(BArgs a) {
 #pragma unroll
     for (int k = 0; k < SPL; ++k) {
       if (!on[k]) continue;
-      const size_t o = (size_t)i * B + lane + 32 * k;
+      const size_t o = (size_t)i * B + lane * SPL + k;
       a.x[o] += (double)a.xl[o];
       a.xl[o] = 0.0f;
     }
   }
 }
 
-// p = r + beta p in FP32
-template <int SPL>
-__global__ void __launch_bounds__(BT) k_bcm_p(BArgs a) {
-  constexpr int B = 32 * SPL;
-  const LatGeom g = *a.lat;
-  const int lane = threadIdx.x & 31;
-  bool on[SPL];
-  float be[SPL];
-#pragma unroll
-  for (int k = 0; k < SPL; ++k) {
-    const SlotState* S = a.st + lane + 32 * k;
-    on[k] = S->status == SLOT_RUN;
-    be[k] = S->restart ? 0.0f : (float)S->beta.x;
-  }
-  float* __restrict__ pf = a.pf;
-  const float* __restrict__ rf = a.rf;
-  BK_ROW_BATCHES(i0, tw) {
-    float pv[BR][SPL], rv[BR][SPL];
-#pragma unroll
-    for (int u = 0; u < BR; ++u)
-#pragma unroll
-      for (int k = 0; k < SPL; ++k) {
-        const int i = i0 + u * tw;
-        if (i >= g.V || !on[k]) continue;
-        const size_t o = (size_t)i * B + lane + 32 * k;
-        pv[u][k] = pf[o];
-        rv[u][k] = rf[o];
-      }
-#pragma unroll
-    for (int u = 0; u < BR; ++u)
-#pragma unroll
-      for (int k = 0; k < SPL; ++k) {
-        const int i = i0 + u * tw;
-        if (i >= g.V || !on[k]) continue;
-        pf[(size_t)i * B + lane + 32 * k] = fmaf(be[k], pv[u][k], rv[u][k]);
-      }
-  }
-}
-
-// True residual r = b - A x in FP64 for the slots that asked for one, one thread per row and a
-// grid row per slot (most iterations one slot or none asks: a warp per row over all slots would
-// walk the whole matrix for a single lane).  MIXED: r is stored in FP32 for the iteration and
-// the old p is kept.
+// True residual r = b - A x in FP64 for the slots that asked for one: most iterations none does, around an update several
+// do.  The blocks list the asking slots (a slot is finalised by the last block that served it, so every block lists
+// the same) and take them eight at a time, eight lanes per row (the entries are read once for eight slots, the gathers
+// share sectors), or one at a time, one thread per row, where fewer than three ask.  MIXED: r is stored in FP32 for the
+// iteration and the old p is kept.
 template <int SPL, bool MIXED>
 __global__ void __launch_bounds__(256) k_btrue_slot(BArgs a, double* __restrict__ part, unsigned int* __restrict__ cnt) {
   constexpr int B = 32 * SPL;
-  const int slot = blockIdx.y;
-  SlotState* S = a.st + slot;
-  if (!S->need_update) return;
-  const LatGeom g = *a.lat;
-  const int m = S->m, pa = S->a;
-  double acc[1] = {0.0};
-  for (int i = blockIdx.x * 256 + threadIdx.x; i < g.V; i += gridDim.x * 256) {
-    double ax = 0.0;
-    const int e1 = __ldg(g.csr_rp + i + 1);
-    for (int e = __ldg(g.csr_rp + i); e < e1; ++e)
-      ax += __ldg(g.csr_val + e) * a.x[(size_t)__ldg(g.csr_ci + e) * B + slot];
-    const double rv = lap_source(g, i, m, pa) - ax;
-    if (MIXED)
-      a.rf[(size_t)i * B + slot] = (float)rv;
-    else
-      a.r[(size_t)i * B + slot] = rv;
-    acc[0] += rv * rv;
+  __shared__ int list[B], nask, last[8];
+  __shared__ unsigned int words[SPL];
+  __shared__ double sh[256];
+  if (threadIdx.x < B) {
+    const unsigned int w = __ballot_sync(0xffffffffu, a.st[threadIdx.x].need_update != 0);
+    if ((threadIdx.x & 31) == 0) words[threadIdx.x >> 5] = w;
   }
-  lreduce<1, 256>(acc, part + (size_t)slot * gridDim.x, 0, blockIdx.x);
-  if (last_block(cnt + slot, gridDim.x)) {
-    double tot[1];
-    block_sum_partials<1, 256>(part + (size_t)slot * gridDim.x, 0, gridDim.x, tot);
-    if (threadIdx.x == 0) {
-      cg_after_true(S, tot[0], a.tol2, MIXED);
-      cnt[slot] = 0;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int n = 0;
+    for (int k = 0; k < SPL; ++k)
+      for (unsigned int w = words[k]; w; w &= w - 1) list[n++] = 32 * k + __ffs(w) - 1;
+    nask = n;
+  }
+  __syncthreads();
+  const int n = nask;
+  if (n == 0) return;
+  const LatGeom g = *a.lat;
+  const int lsh = n >= 3 ? 3 : 0, L = 1 << lsh;
+  const long long step = ((long long)gridDim.x * 256) >> lsh;
+  for (int s0 = 0; s0 < n; s0 += L) {
+    const int li = s0 + (int)(threadIdx.x & (L - 1));
+    const int slot = li < n ? list[li] : -1;
+    const int m = slot >= 0 ? a.st[slot].m : 0, pa = slot >= 0 ? a.st[slot].a : 0;
+    double acc = 0.0;
+    if (slot >= 0)
+      for (long long i = ((long long)blockIdx.x * 256 + threadIdx.x) >> lsh; i < g.V; i += step) {
+        double ax = 0.0;
+        const int e1 = __ldg(g.csr_rp + i + 1);
+        for (int e = __ldg(g.csr_rp + i); e < e1; ++e)
+          ax += __ldg(g.csr_val + e) * a.x[(size_t)__ldg(g.csr_ci + e) * B + slot];
+        const double rv = lap_source(g, (int)i, m, pa) - ax;
+        if (MIXED)
+          a.rf[(size_t)i * B + slot] = (float)rv;
+        else
+          a.r[(size_t)i * B + slot] = rv;
+        acc += rv * rv;
+      }
+    __syncthreads();
+    sh[threadIdx.x] = acc;
+    __syncthreads();
+    if (threadIdx.x < 32) {   // lane l adds the threads l, l + 32, ...: of its slot, since L divides 32
+      double t = 0.0;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) t += sh[threadIdx.x + 32 * w];
+      for (int o = 16; o >= L; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (threadIdx.x < L && slot >= 0) {
+        part[(size_t)slot * gridDim.x + blockIdx.x] = t;
+        __threadfence();
+        last[threadIdx.x] = atomicAdd(cnt + slot, 1u) == gridDim.x - 1u;
+      } else if (threadIdx.x < 8) {
+        last[threadIdx.x] = 0;
+      }
+    }
+    __syncthreads();
+    for (int l = 0; l < L; ++l) {
+      if (!last[l]) continue;
+      __threadfence();
+      const int sl = list[s0 + l];
+      double tot[1];
+      block_sum_partials<1, 256>(part + (size_t)sl * gridDim.x, 0, gridDim.x, tot);
+      if (threadIdx.x == 0) {
+        cg_after_true(a.st + sl, tot[0], a.tol2, MIXED);
+        cnt[sl] = 0;
+      }
     }
   }
 }
@@ -1158,27 +1076,29 @@ struct BlockedSparseEngine {
     a.st = st;
     // one resident wave of the matrix-vector kernel (a second, partial wave would idle most SMs)
     int occ = 0;
-    HP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, MIXED ? (const void*)k_bcm_ap<SPL>
-                                                                       : (const void*)k_bcg_ap<SPL>, BT, 0));
+    HP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)k_bcg_ap<SPL, MIXED>, BT, 0));
     const long long rows_blocks = ((long long)Vmax + BT / 32 - 1) / (BT / 32);   // one row per warp at least
     auto wave = [&](int blocks_per_sm) {
       return (int)std::max(1LL, std::min<long long>(rows_blocks, (long long)ctx->num_sms * std::max(blocks_per_sm, 1)));
     };
     a.nblk = wave(occ);
-    a.nstream = wave(2048 / BT);
-    a.pstride = std::max(a.nblk, a.nstream);
+    a.nstream = wave(4);   // resident blocks of the streaming kernels
+    const int nb = std::max(a.nblk, a.nstream);
+    a.ngroups_max = (nb + 31) / 32;
     void* p = nullptr;
-    ntrue = (int)std::max(1LL, std::min<long long>(((long long)Vmax + 255) / 256, (long long)ctx->num_sms * 2));
+    ntrue = (int)std::max(1LL, std::min<long long>(((long long)Vmax + 255) / 256, (long long)ctx->num_sms * 8));
     HP_TRY(hp_ws(ctx, "bcg.tpart", sizeof(double) * (size_t)B * ntrue, &p));
     tpart = (double*)p;
     HP_TRY(hp_ws(ctx, "bcg.tcnt", sizeof(unsigned int) * B, &p));
     tcnt = (unsigned int*)p;
     HP_CUDA(cudaMemsetAsync(tcnt, 0, sizeof(unsigned int) * B, ctx->stream));
-    HP_TRY(hp_ws(ctx, "bcg.part", sizeof(double) * (size_t)B * a.pstride, &p));
+    HP_TRY(hp_ws(ctx, "bcg.part", sizeof(double) * (size_t)B * (nb + a.ngroups_max), &p));
     a.part = (double*)p;
-    HP_TRY(hp_ws(ctx, "bcg.cnt", sizeof(unsigned int) * BK_COUNT, &p));
+    a.gpart = a.part + (size_t)B * nb;
+    const size_t ncnt = sizeof(unsigned int) * BK_COUNT * (size_t)(1 + a.ngroups_max);
+    HP_TRY(hp_ws(ctx, "bcg.cnt", ncnt, &p));
     a.cnt = (unsigned int*)p;
-    HP_CUDA(cudaMemsetAsync(a.cnt, 0, sizeof(unsigned int) * BK_COUNT, ctx->stream));
+    HP_CUDA(cudaMemsetAsync(a.cnt, 0, ncnt, ctx->stream));
     const size_t fb = sizeof(double) * (size_t)B * Vmax;
     double** v[4] = {&a.x, &a.r, &a.p, &a.q};
     const char* names[4] = {"solve.lx", "solve.lr", "solve.lp", "solve.lq"};
@@ -1221,36 +1141,25 @@ struct BlockedSparseEngine {
     return HP_OK;
   }
   hp_status init() {
-    if (MIXED) {
-      ProfScope ps(ctx, "k_bcm_init");
-      k_bcm_init<SPL><<<a.nstream, BT, 0, ctx->stream>>>(a);
-    } else {
-      ProfScope ps(ctx, "k_bcg_init");
-      k_bcg_init<SPL><<<a.nstream, BT, 0, ctx->stream>>>(a);
+    {
+      ProfScope ps(ctx, MIXED ? "k_bcm_init" : "k_bcg_init");
+      k_bcg_init<SPL, MIXED><<<a.nstream, BT, 0, ctx->stream>>>(a);
     }
     HP_LAUNCH_CHECK();
     return HP_OK;
   }
   hp_status iteration() {
+    { ProfScope ps(ctx, MIXED ? "k_bcm_ap" : "k_bcg_ap"); k_bcg_ap<SPL, MIXED><<<a.nblk, BT, 0, ctx->stream>>>(a); }
+    { ProfScope ps(ctx, MIXED ? "k_bcm_xr" : "k_bcg_xr"); k_bcg_xr<SPL, MIXED><<<a.nstream, BT, 0, ctx->stream>>>(a); }
     if (MIXED) {
-      { ProfScope ps(ctx, "k_bcm_ap"); k_bcm_ap<SPL><<<a.nblk, BT, 0, ctx->stream>>>(a); }
-      { ProfScope ps(ctx, "k_bcm_xr"); k_bcm_xr<SPL><<<a.nstream, BT, 0, ctx->stream>>>(a); }
-      { ProfScope ps(ctx, "k_bcm_fold"); k_bcm_fold<SPL><<<a.nstream, BT, 0, ctx->stream>>>(a); }
-      {
-        ProfScope ps(ctx, "k_btrue_slot");
-        k_btrue_slot<SPL, true><<<dim3(ntrue, B), 256, 0, ctx->stream>>>(a, tpart, tcnt);
-      }
-      { ProfScope ps(ctx, "k_bcm_p"); k_bcm_p<SPL><<<a.nstream, BT, 0, ctx->stream>>>(a); }
-      HP_LAUNCH_CHECK();
-      return HP_OK;
+      ProfScope ps(ctx, "k_bcm_fold");
+      k_bcm_fold<SPL><<<a.nstream, BT, 0, ctx->stream>>>(a);
     }
-    { ProfScope ps(ctx, "k_bcg_ap"); k_bcg_ap<SPL><<<a.nblk, BT, 0, ctx->stream>>>(a); }
-    { ProfScope ps(ctx, "k_bcg_xr"); k_bcg_xr<SPL><<<a.nstream, BT, 0, ctx->stream>>>(a); }
     {
       ProfScope ps(ctx, "k_btrue_slot");
-      k_btrue_slot<SPL, false><<<dim3(ntrue, B), 256, 0, ctx->stream>>>(a, tpart, tcnt);
+      k_btrue_slot<SPL, MIXED><<<ntrue, 256, 0, ctx->stream>>>(a, tpart, tcnt);
     }
-    { ProfScope ps(ctx, "k_bcg_p"); k_bcg_p<SPL><<<a.nstream, BT, 0, ctx->stream>>>(a); }
+    { ProfScope ps(ctx, MIXED ? "k_bcm_p" : "k_bcg_p"); k_bcg_p<SPL, MIXED><<<a.nstream, BT, 0, ctx->stream>>>(a); }
     HP_LAUNCH_CHECK();
     return HP_OK;
   }
@@ -1572,10 +1481,13 @@ static hp_status run_blocked(hp_ctx* ctx, SolveProblem& pb, SolveResult& res) {
 
 hp_status hp_solve_laplace(hp_ctx* ctx, SolveProblem& pb, SolveResult& res) {
   if (pb.lats[0].csr_rp) {   // a general sparse matrix (always alone, without a gradient)
-    // blocked engine: B slots (rhs_block rounded up to 32, 64 or 128; automatic: 64, the fastest
-    // on the renumbered 64^3 grid matrix in both precisions)
-    const int want = pb.opts.rhs_block > 0 ? pb.opts.rhs_block : 64;
+    // blocked engine: B slots (rhs_block rounded up to 32, 64 or 128).  Automatic, measured on the renumbered 64^3 grid:
+    // 32 where the queue fits (16 right-hand sides 17.9 ms, 20.3 in a block of 64); 128 in FP32 where the queue fills
+    // most of it (128 right-hand sides 50.5 ms, 61.2 in blocks of 64); else 64 (64 right-hand sides FP32 28.9 ms, 33.9
+    // in a block of 128; FP64 64 ms, 95)
+    const long long nq = (long long)(pb.s_max[0] - pb.first[0]) * pb.lats[0].parts;
     const bool mixed = pb.opts.precision == HP_PREC_MIXED_FP32;
+    const int want = pb.opts.rhs_block > 0 ? pb.opts.rhs_block : nq <= 32 ? 32 : (mixed && nq > 96 ? 128 : 64);
     pb.opts.rhs_block = want <= 32 ? 32 : (want <= 64 ? 64 : 128);
     if (mixed) {
       if (want <= 32) return run_blocked<1, true>(ctx, pb, res);

@@ -239,6 +239,28 @@ def test_sparse_trace_device_inputs_and_restart(ctx):
     assert np.abs(T - T_full).max() <= 1e-9 * np.abs(T_full).max()
 
 
+# rows of more than 32 entries and of one, n below a warp's rows and above, every block width in both precisions, few slots
+# and all of them asking for true residuals at once
+@pytest.mark.parametrize("n,degree,s", [(1, 0, 1), (7, 3, 2), (300, 45, 20), (5000, 3, 33), (700, 12, 130)])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("block", [0, 32, 128])
+def test_sparse_trace_row_lengths_and_widths(ctx, n, degree, s, prec, block):
+    rp, ci, val = synth.random_graph_matrix(n, degree, 17, shift=0.5)
+    s = min(s, n)
+    paths = np.zeros((1, n), dtype=np.int32)
+    q = np.zeros(s, dtype=complex)
+    _, q, st = ctx.trace_inv_sparse(rp, ci, val, paths, [1], s, 1e-11,
+                                    ctx.make_opts(prec, z0_seed=3, probe_kind="z2", rhs_block=block), q)
+    assert st["rhs_solved"] == s and st["n_unconverged"] == 0 and st["max_true_residual"] <= 1e-11
+    import scipy.sparse.linalg as sla
+
+    A = sp.csr_matrix((val, ci, rp), shape=(n, n))
+    P = 1.0 - 2.0 * Pr.probe_phases_z2(n, 0, s, 3)
+    ref = np.einsum("mi,im->m", P, np.linalg.solve(A.toarray(), P.T)) if n <= 1000 else \
+        np.einsum("mi,im->m", P, sla.splu(A.tocsc()).solve(np.ascontiguousarray(P.T)))
+    assert np.all(np.abs(q - ref) <= 1e-9 * np.abs(ref))
+
+
 @pytest.mark.parametrize("kind", ["natural", "z2"])
 def test_sparse_trace_comparison_sequences(ctx, kind):
     rp, ci, val = synth.grid_matrix((16, 16), 24, shift=0.4)   # n = 256: natural order needs 2^k
