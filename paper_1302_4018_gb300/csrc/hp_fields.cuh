@@ -92,8 +92,8 @@ struct Real_of<PRFF> {
 
 struct FieldPtr {
   void* p;
-  float* nrm;   // half precisions only
-  void* lo;     // float-float fields: the FP32 field of low parts (p holds the high parts)
+  float* nrm;   // half precisions: per-site norm; block fixed point: per-site unit
+  void* lo;     // block fixed point: the FP32 field of remainders (p holds the integers)
 };
 
 template <int PR>
@@ -182,41 +182,93 @@ struct SpinorIO<PR32> {
   }
 };
 
+// Block fixed point, the storage of the float-float solutions: component = (i + l) unit with a 28-bit integer i, an FP32
+// remainder l (|l| < 5) and a power of two `unit` per site (nrm), such that |i| <= 2^27: 49 bits below the site's
+// largest component.  p: int4 [6], lo: float4 [6], in the chunks of SpinorIO<PR32>.  The integers are what the exact hop
+// multiplies (hop_ff).  A component that is not finite makes the unit NaN, and the site with it.
+__device__ __forceinline__ ffl fix_value(int i, float l, float unit) {
+  const float f = (float)(i >> 4) * 16.0f, b = (float)(i & 15) + l;   // both conversions exact
+  const float s = __fadd_rn(f, b), bb = __fsub_rn(s, f);
+  const float e = __fadd_rn(__fsub_rn(f, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  return ffl(s * unit, e * unit);
+}
+
 template <>
 struct SpinorIO<PRFF> {
   static constexpr int NCH = 6;
-  static constexpr int BYTES = 192;
+  static constexpr int BYTES = 196;
   template <typename R>
   __device__ static __forceinline__ void load(FieldPtr f, int Vmax, int slot, int site, cplx<R> (&s)[12]) {
-    cplx<float> h[12], l[12];
-    SpinorIO<PR32>::load(FieldPtr{f.p, nullptr, nullptr}, Vmax, slot, site, h);
-    SpinorIO<PR32>::load(FieldPtr{f.lo, nullptr, nullptr}, Vmax, slot, site, l);
+    const int4* p = (const int4*)f.p + (size_t)slot * 6 * Vmax + site;
+    const float4* q = (const float4*)f.lo + (size_t)slot * 6 * Vmax + site;
+    const float u = f.nrm[(size_t)slot * Vmax + site];
+    int4 h[6];
+    float4 l[6];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) s[k] = {R(ffl(h[k].x, l[k].x)), R(ffl(h[k].y, l[k].y))};
+    for (int k = 0; k < 6; ++k) {
+      h[k] = p[(size_t)k * Vmax];
+      l[k] = q[(size_t)k * Vmax];
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      s[2 * k] = {R(fix_value(h[k].x, l[k].x, u)), R(fix_value(h[k].y, l[k].y, u))};
+      s[2 * k + 1] = {R(fix_value(h[k].z, l[k].z, u)), R(fix_value(h[k].w, l[k].w, u))};
+    }
   }
   template <typename R>
   __device__ static __forceinline__ void load_nc(FieldPtr f, int Vmax, int slot, int site, cplx<R> (&s)[12]) {
-    cplx<float> h[12], l[12];
-    SpinorIO<PR32>::load_nc(FieldPtr{f.p, nullptr, nullptr}, Vmax, slot, site, h);
-    SpinorIO<PR32>::load_nc(FieldPtr{f.lo, nullptr, nullptr}, Vmax, slot, site, l);
-#pragma unroll
-    for (int k = 0; k < 12; ++k) s[k] = {R(ffl(h[k].x, l[k].x)), R(ffl(h[k].y, l[k].y))};
-  }
-  template <typename R>
-  __device__ static __forceinline__ void load_nc_raw(FieldPtr f, int Vmax, int slot, int site, cplx<R> (&s)[12],
-                                                     R& n) {
-    load_nc(f, Vmax, slot, site, s);
-    n = R(1);
+    load(f, Vmax, slot, site, s);
   }
   __device__ static __forceinline__ void store(FieldPtr f, int Vmax, int slot, int site, const cplx<ffl> (&s)[12]) {
-    cplx<float> h[12], l[12];
+    float m = 0.f;
+    bool finite = true;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      h[k] = {s[k].x.hi, s[k].y.hi};
-      l[k] = {s[k].x.lo, s[k].y.lo};
+      const float a = fabsf(s[k].x.hi), b = fabsf(s[k].y.hi);
+      finite = finite && a < INFINITY && b < INFINITY;
+      m = fmaxf(m, fmaxf(a, b));
     }
-    SpinorIO<PR32>::store(FieldPtr{f.p, nullptr, nullptr}, Vmax, slot, site, h);
-    SpinorIO<PR32>::store(FieldPtr{f.lo, nullptr, nullptr}, Vmax, slot, site, l);
+    // m < 2^(E - 126) with E its biased exponent; unit = 2^(E - 126 - 27)
+    const int E = max(__float_as_int(m) >> 23, 37);
+    const float unit = __int_as_float((E - 26) << 23), inv = __int_as_float((280 - E) << 23);
+    int4* p = (int4*)f.p + (size_t)slot * 6 * Vmax + site;
+    float4* q = (float4*)f.lo + (size_t)slot * 6 * Vmax + site;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const ffl v[4] = {s[2 * k].x, s[2 * k].y, s[2 * k + 1].x, s[2 * k + 1].y};
+      int i[4];
+      float l[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float t = v[j].hi * inv;   // exact; an integer already where it has no room for a fraction
+        i[j] = __float2int_rn(t);
+        l[j] = fmaf(v[j].lo, inv, t - (float)i[j]);
+      }
+      p[(size_t)k * Vmax] = make_int4(i[0], i[1], i[2], i[3]);
+      q[(size_t)k * Vmax] = make_float4(l[0], l[1], l[2], l[3]);
+    }
+    f.nrm[(size_t)slot * Vmax + site] = finite ? unit : NAN;
+  }
+  // a site that is zero
+  __device__ static __forceinline__ void store_zero(FieldPtr f, int Vmax, int slot, int site) {
+    int4* p = (int4*)f.p + (size_t)slot * 6 * Vmax + site;
+    float4* q = (float4*)f.lo + (size_t)slot * 6 * Vmax + site;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      p[(size_t)k * Vmax] = make_int4(0, 0, 0, 0);
+      q[(size_t)k * Vmax] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    f.nrm[(size_t)slot * Vmax + site] = 0.f;
+  }
+  // one component
+  __device__ static __forceinline__ double2 component(FieldPtr f, int Vmax, int slot, int site, int comp) {
+    const size_t off = ((size_t)slot * 6 + comp / 2) * Vmax + site;
+    const int4 h = ((const int4*)f.p)[off];
+    const float4 l = ((const float4*)f.lo)[off];
+    const float u = f.nrm[(size_t)slot * Vmax + site];
+    const ffl a = (comp & 1) ? fix_value(h.z, l.z, u) : fix_value(h.x, l.x, u);
+    const ffl b = (comp & 1) ? fix_value(h.w, l.w, u) : fix_value(h.y, l.y, u);
+    return make_double2(ffl_to_double(a), ffl_to_double(b));
   }
 };
 
@@ -405,24 +457,6 @@ struct LinkIO<PR32, 18> {
   }
 };
 
-template <int REC>
-struct LinkIO<PRFF, REC> {
-  static constexpr int BYTES = 144;
-  template <typename R>
-  __device__ static __forceinline__ void load(const LatGeom& g, int mu, int site, cplx<R> (&u)[9]) {
-    const float4* b = g.U32f + (size_t)mu * 4 * g.V + site;
-    const float4* c = g.U32fl + (size_t)mu * 4 * g.V + site;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      float4 v = __ldg(b + (size_t)k * g.V), w = __ldg(c + (size_t)k * g.V);
-      u[2 * k] = {ffl(v.x, w.x), ffl(v.y, w.y)};
-      u[2 * k + 1] = {ffl(v.z, w.z), ffl(v.w, w.w)};
-    }
-    float2 e = __ldg(g.U32g + (size_t)mu * g.V + site), f = __ldg(g.U32gl + (size_t)mu * g.V + site);
-    u[8] = {ffl(e.x, f.x), ffl(e.y, f.y)};
-  }
-};
-
 template <>
 struct LinkIO<PR16, 18> {
   static constexpr int BYTES = 36;
@@ -587,11 +621,11 @@ __device__ __forceinline__ void site_coords(const LatGeom& g, int site, int (&x)
   }
 }
 
-// ---- the float-float hop ----
-// Lazily normalised float-float numbers for the hop sums: the high parts are added with TwoSum
+// ---- the exact hop ----
+// Lazily normalised float-float numbers for the clover products of the exact steps: the high parts are added with TwoSum
 // and products of high parts split exactly with an FMA (TwoProduct), while every rounding error
 // and cross term collects in the low part without renormalising after each operation (the low
-// part stays within a few ulp of the high part over the ~200 terms of a hop, so hi + lo keeps a
+// part stays within a few ulp of the high part over the terms of a block, so hi + lo keeps a
 // 46-bit significand).  One renormalisation per result.
 struct ffz {
   float hi, lo;
@@ -627,17 +661,39 @@ __device__ __forceinline__ int sel4(const int (&v)[4], int mu) {
   return mu == 0 ? v[0] : mu == 1 ? v[1] : mu == 2 ? v[2] : v[3];
 }
 
-// out = hop(in) at `site` in float-float (in: float-float field, HALF: one parity indexed
-// site >> 1).  The eight directions run in a loop that is not unrolled: one copy of the SU(3)
-// product serves all of them (a backward link enters as its adjoint, formed in registers),
-// since the fully unrolled float-float hop overflows the instruction cache.
+// out = hop(in) at `site` to 48 bits (in: block fixed-point field, HALF: one parity indexed site >> 1).
+// The sums run in integers: a link element is 2^-30 (i + l) (30-bit integer and FP32 remainder, prepared once), so the
+// product of the integer parts is one 32 x 32 + 64 bit multiply-add, exact, and only the cross terms i l + l i need FP32
+// (two FMAs, exact to 2^-24 of 2^-28).  That is 3 instructions (4 slots of the FMA pipe) per real multiply-add,
+// 32 of them per clock and SM, where float-float sums take 12 (7.8 per clock and SM); projections and reconstructions
+// are integer adds.  The terms of a direction are shifted to the largest unit of the eight neighbours; the sums stay
+// below 2^63: |i| <= 2^28 after the projection, a row of U has norm 1, so a term is at most sqrt(6) 2^58 and eight of
+// them 2^62.3.  One conversion to float-float per result.
+// 32^3x64, per right-hand side and launch: x_1 0.43 ms, x_2 0.62 ms (float-float sums: 0.59, 0.73 ms).
+// The directions run in a loop that is not unrolled, with one copy of the SU(3) product for all of them (a backward link
+// enters as its adjoint, formed in registers): unrolled, eight copies overflow the instruction cache.
 template <int SPR, int LPR, int REC, bool HALF>
 __device__ __forceinline__ void hop_ff(const LatGeom& g, FieldPtr in, int Vmax, int slot, int site,
                                        const int (&x)[4], const int (&st)[4], cplx<ffl> (&out)[12]) {
-  static_assert(SPR == PRFF && LPR == PRFF, "float-float field and links");
-  cplx<ffz> acc[12];
+  static_assert(SPR == PRFF && LPR == PRFF, "block fixed-point field and links");
+  cplx<long long> acc[12];
+  cplx<float> accl[12];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = {ffz(0), ffz(0)};
+  for (int k = 0; k < 12; ++k) {
+    acc[k] = {0LL, 0LL};
+    accl[k] = {0.f, 0.f};
+  }
+  const float* un = in.nrm + (size_t)slot * Vmax;
+  float umax = 0.f, usum = 0.f;   // the largest unit; the sum is NaN where one is
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    const int L = g.L[mu];
+    const int fw = (x[mu] + 1 == L) ? site - (L - 1) * st[mu] : site + st[mu];
+    const int bw = (x[mu] == 0) ? site + (L - 1) * st[mu] : site - st[mu];
+    const float a = un[HALF ? fw >> 1 : fw], b = un[HALF ? bw >> 1 : bw];
+    umax = fmaxf(umax, fmaxf(a, b));
+    usum += a + b;
+  }
   int L4[4] = {g.L[0], g.L[1], g.L[2], g.L[3]};
 #pragma unroll 1
   for (int d = 0; d < 8; ++d) {
@@ -646,45 +702,110 @@ __device__ __forceinline__ void hop_ff(const LatGeom& g, FieldPtr in, int Vmax, 
     const int xm = sel4(x, mu), sm = sel4(st, mu), L = sel4(L4, mu);
     const int nb = fwd ? ((xm + 1 == L) ? site - (L - 1) * sm : site + sm)
                        : ((xm == 0) ? site + (L - 1) * sm : site - sm);
-    cplx<ffz> u[9], psi[12], h[6], w[6];
+    const int ls = fwd ? site : nb, hn = HALF ? nb >> 1 : nb;
+    cplx<int> h[6];
+    cplx<float> hl[6];
     {
-      cplx<ffl> ul[9], pl[12];
-      LinkIO<LPR, REC>::load(g, mu, fwd ? site : nb, ul);
-      SpinorIO<SPR>::load_nc(in, Vmax, slot, HALF ? nb >> 1 : nb, pl);
+      const int4* p = (const int4*)in.p + (size_t)slot * 6 * Vmax + hn;
+      const float4* q = (const float4*)in.lo + (size_t)slot * 6 * Vmax + hn;
+      cplx<int> xi[12];
+      cplx<float> xl[12];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        const int4 v = __ldg(p + (size_t)k * Vmax);
+        const float4 w = __ldg(q + (size_t)k * Vmax);
+        xi[2 * k] = {v.x, v.y};
+        xi[2 * k + 1] = {v.z, v.w};
+        xl[2 * k] = {w.x, w.y};
+        xl[2 * k + 1] = {w.z, w.w};
+      }
+      switch (d) {
+        case 0: project<0, -1>(xi, h); project<0, -1>(xl, hl); break;
+        case 1: project<0, 1>(xi, h); project<0, 1>(xl, hl); break;
+        case 2: project<1, -1>(xi, h); project<1, -1>(xl, hl); break;
+        case 3: project<1, 1>(xi, h); project<1, 1>(xl, hl); break;
+        case 4: project<2, -1>(xi, h); project<2, -1>(xl, hl); break;
+        case 5: project<2, 1>(xi, h); project<2, 1>(xl, hl); break;
+        case 6: project<3, -1>(xi, h); project<3, -1>(xl, hl); break;
+        default: project<3, 1>(xi, h); project<3, 1>(xl, hl); break;
+      }
+    }
+    cplx<int> ui[9];
+    cplx<float> ul[9];
+    {
+      const int4* p = g.U32i + (size_t)mu * 4 * g.V + ls;
+      const float4* q = g.U32fl + (size_t)mu * 4 * g.V + ls;
+      cplx<int> a[9];
+      cplx<float> b[9];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int4 v = __ldg(p + (size_t)k * g.V);
+        const float4 w = __ldg(q + (size_t)k * g.V);
+        a[2 * k] = {v.x, v.y};
+        a[2 * k + 1] = {v.z, v.w};
+        b[2 * k] = {w.x, w.y};
+        b[2 * k + 1] = {w.z, w.w};
+      }
+      const int2 v = __ldg(g.U32gi + (size_t)mu * g.V + ls);
+      const float2 w = __ldg(g.U32gl + (size_t)mu * g.V + ls);
+      a[8] = {v.x, v.y};
+      b[8] = {w.x, w.y};
 #pragma unroll
       for (int r = 0; r < 3; ++r)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const cplx<ffl> e = fwd ? ul[3 * r + c] : ul[3 * c + r];   // U or U^dagger
-          u[3 * r + c] = {ffz(e.x.hi, e.x.lo), fwd ? ffz(e.y.hi, e.y.lo) : ffz(-e.y.hi, -e.y.lo)};
+        for (int c = 0; c < 3; ++c) {   // U or U^dagger
+          ui[3 * r + c] = fwd ? a[3 * r + c] : cplx<int>{a[3 * c + r].x, -a[3 * c + r].y};
+          ul[3 * r + c] = fwd ? b[3 * r + c] : cplx<float>{b[3 * c + r].x, -b[3 * c + r].y};
         }
+    }
+    const int sh = min(63, (__float_as_int(umax) - __float_as_int(un[hn])) >> 23);
+    const float sc = __int_as_float((127 - sh) << 23);
+    cplx<long long> w[6];
+    cplx<float> wl[6];
 #pragma unroll
-      for (int k = 0; k < 12; ++k) psi[k] = {ffz(pl[k].x.hi, pl[k].x.lo), ffz(pl[k].y.hi, pl[k].y.lo)};
-    }
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        long long ax = 0, ay = 0;
+        float fx = 0.f, fy = 0.f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const int a = ui[3 * r + c].x, b = ui[3 * r + c].y, hx = h[3 * s + c].x, hy = h[3 * s + c].y;
+          const float af = (float)a, bf = (float)b, al = ul[3 * r + c].x, bl = ul[3 * r + c].y;
+          const float hfx = (float)hx, hfy = (float)hy, hlx = hl[3 * s + c].x, hly = hl[3 * s + c].y;
+          ax += (long long)a * hx;
+          ax += (long long)(-b) * hy;
+          ay += (long long)a * hy;
+          ay += (long long)b * hx;
+          fx = fmaf(af, hlx, fmaf(al, hfx, fmaf(-bf, hly, fmaf(-bl, hfy, fx))));
+          fy = fmaf(af, hly, fmaf(al, hfy, fmaf(bf, hlx, fmaf(bl, hfx, fy))));
+        }
+        w[3 * s + r] = {ax >> sh, ay >> sh};
+        wl[3 * s + r] = {fx * sc, fy * sc};
+      }
     switch (d) {
-      case 0: project<0, -1>(psi, h); break;
-      case 1: project<0, 1>(psi, h); break;
-      case 2: project<1, -1>(psi, h); break;
-      case 3: project<1, 1>(psi, h); break;
-      case 4: project<2, -1>(psi, h); break;
-      case 5: project<2, 1>(psi, h); break;
-      case 6: project<3, -1>(psi, h); break;
-      default: project<3, 1>(psi, h); break;
-    }
-    su3_mul<ffz, false>(u, h, w);
-    switch (d) {
-      case 0: accumulate<0, -1>(acc, w); break;
-      case 1: accumulate<0, 1>(acc, w); break;
-      case 2: accumulate<1, -1>(acc, w); break;
-      case 3: accumulate<1, 1>(acc, w); break;
-      case 4: accumulate<2, -1>(acc, w); break;
-      case 5: accumulate<2, 1>(acc, w); break;
-      case 6: accumulate<3, -1>(acc, w); break;
-      default: accumulate<3, 1>(acc, w); break;
+      case 0: accumulate<0, -1>(acc, w); accumulate<0, -1>(accl, wl); break;
+      case 1: accumulate<0, 1>(acc, w); accumulate<0, 1>(accl, wl); break;
+      case 2: accumulate<1, -1>(acc, w); accumulate<1, -1>(accl, wl); break;
+      case 3: accumulate<1, 1>(acc, w); accumulate<1, 1>(accl, wl); break;
+      case 4: accumulate<2, -1>(acc, w); accumulate<2, -1>(accl, wl); break;
+      case 5: accumulate<2, 1>(acc, w); accumulate<2, 1>(accl, wl); break;
+      case 6: accumulate<3, -1>(acc, w); accumulate<3, -1>(accl, wl); break;
+      default: accumulate<3, 1>(acc, w); accumulate<3, 1>(accl, wl); break;
     }
   }
+  // (acc + accl) 2^-30 umax: 24 leading bits, the 24 below them, and the rest with the cross terms
+  const float scale = umax * 0x1p-30f + 0.0f * usum;
+  auto value = [scale](long long a, float l) {
+    const float top = (float)(int)(a >> 39) * 0x1p39f;
+    const long long rest = a & 0x7fffffffffLL;
+    const float low = fmaf((float)(int)(rest >> 15), 0x1p15f, (float)(int)(rest & 0x7fff) + l);
+    const float s = __fadd_rn(top, low), bb = __fsub_rn(s, top);
+    const float e = __fadd_rn(__fsub_rn(top, __fsub_rn(s, bb)), __fsub_rn(low, bb));
+    return ffl(s * scale, e * scale);
+  };
 #pragma unroll
-  for (int k = 0; k < 12; ++k) out[k] = {ffl_of(acc[k].x), ffl_of(acc[k].y)};
+  for (int k = 0; k < 12; ++k) out[k] = {value(acc[k].x, accl[k].x), value(acc[k].y, accl[k].y)};
 }
 
 // hop = sum_mu [(1 - g_mu) U_mu(x) psi(x+mu) + (1 + g_mu) U_mu(x-mu)^H psi(x-mu)]
@@ -695,8 +816,7 @@ __device__ __forceinline__ void wilson_hop(const LatGeom& g, FieldPtr in, int Vm
   for (int k = 0; k < 12; ++k) acc[k] = {0, 0};
   if constexpr (is_ffl<R>::value) {
     hop_ff<SPR, LPR, 12, false>(g, in, Vmax, slot, site, x, st, acc);
-    return;
-  }
+  } else {
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
     const int L = g.L[mu];
@@ -725,6 +845,7 @@ __device__ __forceinline__ void wilson_hop(const LatGeom& g, FieldPtr in, int Vm
     if (mu == 1) accumulate<1, 1>(acc, w);
     if (mu == 2) accumulate<2, 1>(acc, w);
     if (mu == 3) accumulate<3, 1>(acc, w);
+  }
   }
 }
 

@@ -42,7 +42,8 @@ void hp_set_error(const char* fmt, ...);
   } while (0)
 
 // -------------------------------------------------------------- precisions
-// PRFF: float-float (an unevaluated sum hi + lo of two FP32 numbers, 48-bit significand)
+// PRFF: float-float (an unevaluated sum hi + lo of two FP32 numbers, 48-bit significand), fields of it stored in block
+// fixed point (hp_fields.cuh)
 enum { PR64 = 0, PR32 = 1, PR16 = 2, PRB16 = 3, PRFF = 4 };
 
 // ---------------------------------------------------------- lattice (device)
@@ -92,8 +93,10 @@ struct LatGeom {
   const float2* U32g;         // [4][V]     entry 8
   const uint4* U16f;          // [4][2][V]  entries 0-7 of the full link, binary16
   const unsigned int* U16g;   // [4][V]     entry 8
-  const float4* U32fl;        // [4][4][V]  low parts (u - (float)u) of entries 0-7, float-float links
-  const float2* U32gl;        // [4][V]     low part of entry 8
+  const int4* U32i;           // [4][4][V]  fixed-point links of the exact steps: u = 2^-30 (i + l), i an integer (0-7)
+  const int2* U32gi;          // [4][V]     entry 8
+  const float4* U32fl;        // [4][4][V]  their remainders l, |l| <= 1/2
+  const float2* U32gl;        // [4][V]     entry 8
   // clover term: A(x) = (1 + m + mu(x)) + C(x) (Wilson diagonal plus the Sheikholeslami-Wohlert
   // term) as two Hermitian 6x6 blocks per site (spins 0-1 and 2-3: C commutes with gamma_5),
   // each packed as 6 real diagonal entries then the 15 entries above the diagonal (row-major)

@@ -15,7 +15,8 @@
 __global__ void k_links_convert(const double2* __restrict__ in, int V, double2* __restrict__ U64,
                                 float4* __restrict__ U32, uint2* __restrict__ U16, float4* __restrict__ U32f,
                                 float2* __restrict__ U32g, uint4* __restrict__ U16f, unsigned int* __restrict__ U16g,
-                                float4* __restrict__ U32fl, float2* __restrict__ U32gl) {
+                                float4* __restrict__ U32fl, float2* __restrict__ U32gl, int4* __restrict__ U32i,
+                                int2* __restrict__ U32gi) {
   const long long total = 4LL * V;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
@@ -49,13 +50,28 @@ __global__ void k_links_convert(const double2* __restrict__ in, int V, double2* 
             make_float4((float)u[2 * k].x, (float)u[2 * k].y, (float)u[2 * k + 1].x, (float)u[2 * k + 1].y);
       U32g[(size_t)mu * V + site] = make_float2((float)u[8].x, (float)u[8].y);
     }
-    if (U32fl) {   // low parts of the float-float links: u - (float)u, exact in FP32
-      auto lo = [](double v) { return (float)(v - (double)(float)v); };
+    if (U32fl) {   // fixed-point links: 2^30 u = i + l, from the FP32 parts of u (u - (float)u is exact in FP32)
+      int ii[18];
+      float ll[18];
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        U32fl[((size_t)mu * 4 + k) * V + site] =
-            make_float4(lo(u[2 * k].x), lo(u[2 * k].y), lo(u[2 * k + 1].x), lo(u[2 * k + 1].y));
-      U32gl[(size_t)mu * V + site] = make_float2(lo(u[8].x), lo(u[8].y));
+      for (int k = 0; k < 9; ++k)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const double v = c ? u[k].y : u[k].x;
+          const float hi = (float)v, t = hi * 0x1p30f;
+          const int a = __float2int_rn(t);
+          const float r = fmaf((float)(v - (double)hi), 0x1p30f, t - (float)a);   // |r| <= 33
+          const int b = __float2int_rn(r);
+          ii[2 * k + c] = a + b;
+          ll[2 * k + c] = r - (float)b;
+        }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        U32i[((size_t)mu * 4 + k) * V + site] = make_int4(ii[4 * k], ii[4 * k + 1], ii[4 * k + 2], ii[4 * k + 3]);
+        U32fl[((size_t)mu * 4 + k) * V + site] = make_float4(ll[4 * k], ll[4 * k + 1], ll[4 * k + 2], ll[4 * k + 3]);
+      }
+      U32gi[(size_t)mu * V + site] = make_int2(ii[16], ii[17]);
+      U32gl[(size_t)mu * V + site] = make_float2(ll[16], ll[17]);
     }
     if (U16f) {
 #pragma unroll
@@ -111,7 +127,7 @@ hp_status hp_prepare_wilson(hp_ctx* ctx, const hp_operator* op, LatGeom* g, cons
   // read once, by the conversion below: pinned host links stream in over the host link directly
   HP_TRY(hp_stream_view(ctx, op->links, sizeof(double) * 72 * V, (base + ".links_in").c_str(), &src));
   void *u64 = nullptr, *u32 = nullptr, *u16 = nullptr, *u32f = nullptr, *u32g = nullptr, *u16f = nullptr,
-       *u16g = nullptr, *u32fl = nullptr, *u32gl = nullptr;
+       *u16g = nullptr, *u32fl = nullptr, *u32gl = nullptr, *u32i = nullptr, *u32gi = nullptr;
   HP_TRY(hp_ws(ctx, (base + ".U64").c_str(), sizeof(double2) * 36 * V, &u64));   // always: true residual
   if (need_prec & (1 << PR32)) {
     HP_TRY(hp_ws(ctx, (base + ".U32").c_str(), sizeof(float4) * 12 * V, &u32));
@@ -119,6 +135,8 @@ hp_status hp_prepare_wilson(hp_ctx* ctx, const hp_operator* op, LatGeom* g, cons
     HP_TRY(hp_ws(ctx, (base + ".U32g").c_str(), sizeof(float2) * 4 * V, &u32g));
     HP_TRY(hp_ws(ctx, (base + ".U32fl").c_str(), sizeof(float4) * 16 * V, &u32fl));
     HP_TRY(hp_ws(ctx, (base + ".U32gl").c_str(), sizeof(float2) * 4 * V, &u32gl));
+    HP_TRY(hp_ws(ctx, (base + ".U32i").c_str(), sizeof(int4) * 16 * V, &u32i));
+    HP_TRY(hp_ws(ctx, (base + ".U32gi").c_str(), sizeof(int2) * 4 * V, &u32gi));
   }
   if (need_prec & (1 << PR16)) {
     HP_TRY(hp_ws(ctx, (base + ".U16").c_str(), sizeof(uint2) * 12 * V, &u16));
@@ -129,7 +147,7 @@ hp_status hp_prepare_wilson(hp_ctx* ctx, const hp_operator* op, LatGeom* g, cons
     ProfScope ps(ctx, "k_links_convert");
     k_links_convert<<<blocks_for(ctx, 4LL * V, 256), 256, 0, ctx->stream>>>(
         (const double2*)src, (int)V, (double2*)u64, (float4*)u32, (uint2*)u16, (float4*)u32f, (float2*)u32g,
-        (uint4*)u16f, (unsigned int*)u16g, (float4*)u32fl, (float2*)u32gl);
+        (uint4*)u16f, (unsigned int*)u16g, (float4*)u32fl, (float2*)u32gl, (int4*)u32i, (int2*)u32gi);
   }
   HP_LAUNCH_CHECK();
   g->U64 = (const double2*)u64;
@@ -141,6 +159,8 @@ hp_status hp_prepare_wilson(hp_ctx* ctx, const hp_operator* op, LatGeom* g, cons
   g->U16g = (const unsigned int*)u16g;
   g->U32fl = (const float4*)u32fl;
   g->U32gl = (const float2*)u32gl;
+  g->U32i = (const int4*)u32i;
+  g->U32gi = (const int2*)u32gi;
   return hp_prepare_clover(ctx, op, g, tag);
 }
 

@@ -84,7 +84,7 @@ struct WArgs {
   FieldPtr r, rh, p, v, s, t, e;
   FieldPtr rg;           // group-updated residual (FP32), mixed precision only
   double2* x;            // FP64 solution [slot][12][Vmax] (FP64 solves)
-  FieldPtr xff;          // float-float solution (hi, lo FP32 fields), mixed precision
+  FieldPtr xff;          // solution in block fixed point (integers, remainders, units), mixed precision
   double tol2, delta2, epsx2;
   int maxiter;
   // even-odd: Krylov fields live on the odd sites (half-site index = site >> 1)
@@ -92,7 +92,7 @@ struct WArgs {
   FieldPtr mid;          // even-site intermediate of the Schur operator (iteration precision)
   FieldPtr mid32;        // even-site intermediate of group updates (FP32)
   double2* xe;           // even-site solution, FP64 solves
-  FieldPtr xeff;         // even-site solution, float-float (mixed)
+  FieldPtr xeff;         // even-site solution, block fixed point (mixed)
 };
 
 #define SLOT_PREAMBLE(COND)                                        \
@@ -390,11 +390,7 @@ __global__ void __launch_bounds__(NT) k_bicg_init(WArgs a) {
     if (SPR == PR64) {
       SpinorIO<PR64>::store(FieldPtr{a.x, nullptr, nullptr}, a.Vmax, slot, site, z);
     } else {
-      cplx<float> zf[12];
-#pragma unroll
-      for (int k = 0; k < 12; ++k) zf[k] = {0.f, 0.f};
-      SpinorIO<PR32>::store(FieldPtr{a.xff.p, nullptr, nullptr}, a.Vmax, slot, site, zf);
-      SpinorIO<PR32>::store(FieldPtr{a.xff.lo, nullptr, nullptr}, a.Vmax, slot, site, zf);
+      SpinorIO<PRFF>::store_zero(a.xff, a.Vmax, slot, site);
     }
     {
       cplx<typename Real_of<EPR>::T> ze[12];
@@ -620,7 +616,7 @@ __global__ void __launch_bounds__(NT) k_grp_update(WArgs a) {
 }
 
 // ---- reliable update, part 1: x += e ; e = 0
-// FP64 solves keep x in FP64; mixed solves keep x in float-float (hi, lo FP32 fields)
+// FP64 solves keep x in FP64; mixed solves keep x in block fixed point (float-float values, SpinorIO<PRFF>)
 template <int SPR, int EPR, int NT>
 __global__ void __launch_bounds__(NT) k_ru_accum(WArgs a) {
   SLOT_PREAMBLE(S->need_update)
@@ -678,7 +674,7 @@ __device__ __forceinline__ void ru_finalize(WArgs& a, SlotState* S, const double
 
 // ---- reliable update, part 2: the true residual r = b - D x, stored in the iteration precision
 // (and in the FP32 group residual).  FP64 solves: FP64 links and arithmetic.  Mixed solves:
-// float-float links, solution and arithmetic on the FP32 pipes (48-bit significand: the
+// fixed-point links and solution, the hop in integer multiply-adds (48 bits: the
 // rounding error of b - D x is ~1e-14 ||b||, far below any tolerance the solver certifies).
 template <int SPR, int NT>
 __global__ void __launch_bounds__(NT, 3) k_ru_residual(WArgs a) {
@@ -808,10 +804,7 @@ __global__ void __launch_bounds__(NT) k_bicg_p(WArgs a) {
 // one component of the converged solution in FP64 (from FP64 or float-float storage)
 __device__ __forceinline__ double2 solution_component(const WArgs& a, int slot, int site, int comp) {
   if (a.x) return a.x[((size_t)slot * 12 + comp) * a.Vmax + site];
-  const size_t off = ((size_t)slot * 6 + comp / 2) * a.Vmax + site;
-  const float4 h = ((const float4*)a.xff.p)[off], l = ((const float4*)a.xff.lo)[off];
-  return (comp & 1) ? make_double2((double)h.z + (double)l.z, (double)h.w + (double)l.w)
-                    : make_double2((double)h.x + (double)l.x, (double)h.y + (double)l.y);
+  return SpinorIO<PRFF>::component(a.xff, a.Vmax, slot, site, comp);
 }
 
 template <int NT>
@@ -897,7 +890,7 @@ __device__ __forceinline__ int eo_site(const LatGeom& g, int h, int par, int (&x
 template <int SPR, int LPR, int REC, typename R>
 __device__ __forceinline__ void eo_hop(const LatGeom& g, FieldPtr in, int Vs, int slot, int site, const int (&x)[4],
                                        const int (&st)[4], R sc, cplx<R> (&acc)[12]) {
-  if constexpr (is_ffl<R>::value) {   // float-float fields (norm 1): acc += sc hop
+  if constexpr (is_ffl<R>::value) {   // block fixed-point fields: acc += sc hop
     cplx<ffl> t[12];
     hop_ff<SPR, LPR, REC, true>(g, in, Vs, slot, site, x, st, t);
 #pragma unroll
@@ -905,8 +898,7 @@ __device__ __forceinline__ void eo_hop(const LatGeom& g, FieldPtr in, int Vs, in
       acc[k].x = fma(sc, t[k].x, acc[k].x);
       acc[k].y = fma(sc, t[k].y, acc[k].y);
     }
-    return;
-  }
+  } else {
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
     const int L = g.L[mu];
@@ -936,6 +928,7 @@ __device__ __forceinline__ void eo_hop(const LatGeom& g, FieldPtr in, int Vs, in
     if (mu == 1) accumulate_s<1, 1>(acc, w, sc * n);
     if (mu == 2) accumulate_s<2, 1>(acc, w, sc * n);
     if (mu == 3) accumulate_s<3, 1>(acc, w, sc * n);
+  }
   }
 }
 
@@ -1134,7 +1127,7 @@ __global__ void __launch_bounds__(NT, EO_ODD_MINB(SIN, REC)) k_eo_odd(WArgs a, F
 // spills at 168; without spills it runs 13% faster)
 #define EO_X_MINB 3
 #define EO_X2_MINB 2
-// ---- exact step 1: x_e = d_e^-1 (b_e + k hop(x_o))   (FP64 or float-float)
+// ---- exact step 1: x_e = d_e^-1 (b_e + k hop(x_o))   (FP64, or 48 bits on fixed-point fields)
 template <int PX, int NT>
 __global__ void __launch_bounds__(NT, EO_X_MINB) k_eo_x1(WArgs a, int nslots) {
   EO_SLOTS_BEGIN(MASK_EXACT, true)
@@ -1292,11 +1285,7 @@ __global__ void __launch_bounds__(NT) k_eo_init(WArgs a, int nslots) {
     }
     if ((par & 1) == 0) {           // odd sites carry the Krylov vectors
       if (SPR != PR64) {            // x_e = 0 until the first exact step (the mixed start skips it)
-        cplx<float> z[12];
-#pragma unroll
-        for (int k = 0; k < 12; ++k) z[k] = {0.f, 0.f};
-        SpinorIO<PR32>::store(FieldPtr{a.xeff.p, nullptr, nullptr}, a.Vmax, slot, h, z);
-        SpinorIO<PR32>::store(FieldPtr{a.xeff.lo, nullptr, nullptr}, a.Vmax, slot, h, z);
+        SpinorIO<PRFF>::store_zero(a.xeff, a.Vmax, slot, h);
       }
       continue;
     }
@@ -1310,11 +1299,7 @@ __global__ void __launch_bounds__(NT) k_eo_init(WArgs a, int nslots) {
       for (int k = 0; k < 12; ++k) z[k] = {0.0, 0.0};
       SpinorIO<PR64>::store(FieldPtr{a.x, nullptr, nullptr}, a.Vmax, slot, h, z);
     } else {
-      cplx<float> z[12];
-#pragma unroll
-      for (int k = 0; k < 12; ++k) z[k] = {0.f, 0.f};
-      SpinorIO<PR32>::store(FieldPtr{a.xff.p, nullptr, nullptr}, a.Vmax, slot, h, z);
-      SpinorIO<PR32>::store(FieldPtr{a.xff.lo, nullptr, nullptr}, a.Vmax, slot, h, z);
+      SpinorIO<PRFF>::store_zero(a.xff, a.Vmax, slot, h);
     }
   }
   reduce_partials<double, 1, NT>(acc, part, a.gy);
@@ -1428,11 +1413,7 @@ __device__ __forceinline__ double2 eo_solution_component(const WArgs& a, int slo
     const double2* f = par ? a.x : a.xe;
     return f[((size_t)slot * 12 + comp) * a.Vmax + h];
   }
-  const FieldPtr f = par ? a.xff : a.xeff;
-  const size_t off = ((size_t)slot * 6 + comp / 2) * a.Vmax + h;
-  const float4 hi = ((const float4*)f.p)[off], lo = ((const float4*)f.lo)[off];
-  return (comp & 1) ? make_double2((double)hi.z + (double)lo.z, (double)hi.w + (double)lo.w)
-                    : make_double2((double)hi.x + (double)lo.x, (double)hi.y + (double)lo.y);
+  return SpinorIO<PRFF>::component(par ? a.xff : a.xeff, a.Vmax, slot, h, comp);
 }
 
 __device__ __forceinline__ int site_parity(const LatGeom& g, int site) {
@@ -1590,14 +1571,18 @@ struct WilsonEngine {
         a.xe = (double2*)p;
       }
     } else {   // float-float solution
-      HP_TRY(alloc_field(ctx, "solve.xhi", PR32, ns, Vmax, &a.xff));
+      HP_TRY(alloc_field(ctx, "solve.xhi", PR32, ns, Vmax, &a.xff));   // integers
       FieldPtr lo;
-      HP_TRY(alloc_field(ctx, "solve.xlo", PR32, ns, Vmax, &lo));
+      HP_TRY(alloc_field(ctx, "solve.xlo", PR32, ns, Vmax, &lo));      // remainders
       a.xff.lo = lo.p;
+      HP_TRY(hp_ws(ctx, "solve.xunit", sizeof(float) * (size_t)ns * Vmax, &p));
+      a.xff.nrm = (float*)p;
       if (eo) {
         HP_TRY(alloc_field(ctx, "solve.xehi", PR32, ns, Vmax, &a.xeff));
         HP_TRY(alloc_field(ctx, "solve.xelo", PR32, ns, Vmax, &lo));
         a.xeff.lo = lo.p;
+        HP_TRY(hp_ws(ctx, "solve.xeunit", sizeof(float) * (size_t)ns * Vmax, &p));
+        a.xeff.nrm = (float*)p;
       }
     }
     if (eo) {

@@ -719,6 +719,27 @@ def test_laplacian_clusters_bounds_gradient_deflation(ctx, hp):
         assert np.allclose(a, b, rtol=2e-9, atol=0)
 
 
+# the exact steps on block fixed-point fields whose sites differ by 10^3 in magnitude (a mass field over three decades, which
+# the FP64 solver converges on too), even-odd and full lattice: the residual of the returned solutions, recomputed by
+# the oracle in FP64.  The returned FP64 values round a 49-bit fixed-point solution, so 2^-49 |D| |x| / |b| <= 1e-13 comes on top.
+@pytest.mark.parametrize("dims,prec,eo", [((4, 4, 4, 4), "fp16", 1), ((3, 5, 4, 2), "fp32", 0), ((6, 4, 2, 8), "bf16", 1)])
+def test_exact_residual_with_sites_of_different_magnitude(ctx, hp, dims, prec, eo):
+    V = int(np.prod(dims))
+    U = synth.gauge_links(dims, 0.4, 41)
+    mu = 10.0 ** np.random.default_rng(5).uniform(0, 3, V)
+    op = ctx.make_operator(hp.OP_WILSON, 0.0, 0.12, links_dev(U), dev(mu))
+    x = torch.empty(12 * V * 24, dtype=torch.float64, device="cuda:0")
+    _, _, st = ctx.trace_inv_solutions(op, dims, 1, 1e-10, ctx.make_opts(prec, z0_seed=7, even_odd=eo), x)
+    assert st["max_true_residual"] <= 1e-10
+    X = x.cpu().numpy().view(np.complex128).reshape(12, V, 4, 3)
+    z = E.probe_vectors(dims, 0, 1, 7)[0]
+    for a in range(12):
+        b = np.zeros((V, 12), dtype=complex)
+        b[:, a] = z
+        r = b - O.wilson_apply(X[a], U, dims, 0.12, 0.0, mu).reshape(V, 12)
+        assert np.linalg.norm(r) <= (1e-10 + 1e-13) * np.linalg.norm(b)
+
+
 # ------------------------------------------------------------------ the comparison sequences (Section 5.2)
 @pytest.mark.parametrize("kind,dims,seed", [("natural", (8, 8, 8, 8), 0), ("natural", (2, 4, 8), 11),
                                             ("natural", (1024,), 3), ("z2", (4, 4, 4, 4), 12345),
