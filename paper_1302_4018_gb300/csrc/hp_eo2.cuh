@@ -399,8 +399,8 @@ __device__ __forceinline__ void hop_dir2(const LatGeom& g, FieldPtr in, int Vmax
   }
 }
 
-// acc += scale * hop(in) at full site `site` (parity par of the output; `in` holds the other parity)
-template <int SPR, int LPR>
+// acc += scale * hop(in) at full site `site` (HALF: `in` holds the other parity, numbered site >> 1)
+template <int SPR, int LPR, bool HALF = true>
 __device__ __forceinline__ void eo_hop2(const LatGeom& g, FieldPtr in, int Vmax, int sa, int sb, int site,
                                         const int (&x)[4], const int (&st)[4], f2 scale, c2 (&acc)[12]) {
 #pragma unroll
@@ -409,17 +409,17 @@ __device__ __forceinline__ void eo_hop2(const LatGeom& g, FieldPtr in, int Vmax,
     const int fw = (x[mu] + 1 == L) ? site - (L - 1) * st[mu] : site + st[mu];
     const int bw = (x[mu] == 0) ? site + (L - 1) * st[mu] : site - st[mu];
     if (mu == 0) {
-      hop_dir2<SPR, LPR, 0, -1>(g, in, Vmax, sa, sb, fw >> 1, site, scale, acc);
-      hop_dir2<SPR, LPR, 0, 1>(g, in, Vmax, sa, sb, bw >> 1, bw, scale, acc);
+      hop_dir2<SPR, LPR, 0, -1>(g, in, Vmax, sa, sb, HALF ? fw >> 1 : fw, site, scale, acc);
+      hop_dir2<SPR, LPR, 0, 1>(g, in, Vmax, sa, sb, HALF ? bw >> 1 : bw, bw, scale, acc);
     } else if (mu == 1) {
-      hop_dir2<SPR, LPR, 1, -1>(g, in, Vmax, sa, sb, fw >> 1, site, scale, acc);
-      hop_dir2<SPR, LPR, 1, 1>(g, in, Vmax, sa, sb, bw >> 1, bw, scale, acc);
+      hop_dir2<SPR, LPR, 1, -1>(g, in, Vmax, sa, sb, HALF ? fw >> 1 : fw, site, scale, acc);
+      hop_dir2<SPR, LPR, 1, 1>(g, in, Vmax, sa, sb, HALF ? bw >> 1 : bw, bw, scale, acc);
     } else if (mu == 2) {
-      hop_dir2<SPR, LPR, 2, -1>(g, in, Vmax, sa, sb, fw >> 1, site, scale, acc);
-      hop_dir2<SPR, LPR, 2, 1>(g, in, Vmax, sa, sb, bw >> 1, bw, scale, acc);
+      hop_dir2<SPR, LPR, 2, -1>(g, in, Vmax, sa, sb, HALF ? fw >> 1 : fw, site, scale, acc);
+      hop_dir2<SPR, LPR, 2, 1>(g, in, Vmax, sa, sb, HALF ? bw >> 1 : bw, bw, scale, acc);
     } else {
-      hop_dir2<SPR, LPR, 3, -1>(g, in, Vmax, sa, sb, fw >> 1, site, scale, acc);
-      hop_dir2<SPR, LPR, 3, 1>(g, in, Vmax, sa, sb, bw >> 1, bw, scale, acc);
+      hop_dir2<SPR, LPR, 3, -1>(g, in, Vmax, sa, sb, HALF ? fw >> 1 : fw, site, scale, acc);
+      hop_dir2<SPR, LPR, 3, 1>(g, in, Vmax, sa, sb, HALF ? bw >> 1 : bw, bw, scale, acc);
     }
   }
 }
@@ -509,7 +509,8 @@ __device__ __forceinline__ void reduce_pair(const float (&v)[2][NQ], double* par
 
 // ---- odd sites: out = A_o in - k^2 hop(mid) with the solver epilogues, two right-hand sides per thread
 //   EPI_V: v = S p, (r^, v), alpha       EPI_T: t = S s, (t, s), (t, t), omega
-template <int SPR, int LPR, int NT, int MINB, int EPI, bool CL, int TPB>
+// FULL: the same steps of the full-lattice iteration, out = A in - k hop(in) on every site
+template <int SPR, int LPR, int NT, int MINB, int EPI, bool CL, int TPB, bool FULL = false>
 __global__ void __launch_bounds__(NT, MINB) k_eo2_odd(WArgs a, FieldPtr in, FieldPtr mid, FieldPtr out, int nslots) {
   // TPB consecutive tiles per block (one reduction per TPB tiles; consecutive, so that the sweep
   // of the lattice stays one front and the neighbours of a tile are still in L2)
@@ -521,7 +522,7 @@ __global__ void __launch_bounds__(NT, MINB) k_eo2_odd(WArgs a, FieldPtr in, Fiel
   const int sa = on0 ? s0 : s1, sb = (on0 && on1) ? s1 : sa;
   const bool two = sb != sa;
   const LatGeom g = a.lats[a.st[sa].lat];
-  const int nsite = g.V >> 1;
+  const int nsite = FULL ? g.V : g.V >> 1;
   const int ntiles = (nsite + NT - 1) / NT;
   const int nchunks = (ntiles + TPB - 1) / TPB;
   if ((int)blockIdx.y >= nchunks) return;
@@ -537,12 +538,14 @@ __global__ void __launch_bounds__(NT, MINB) k_eo2_odd(WArgs a, FieldPtr in, Fiel
   for (int L = 0; L < 2; ++L)
 #pragma unroll
     for (int q = 0; q < NQ; ++q) dots[L][q] = 0.f;
-  const float mk2 = -(float)(g.kappa * g.kappa);
+  const float mk2 = FULL ? -(float)g.kappa : -(float)(g.kappa * g.kappa);
   for (int tile = blockIdx.y * TPB; tile < min(ntiles, (int)(blockIdx.y + 1) * TPB); ++tile) {
     const int h = tile * NT + threadIdx.x;
     if (h >= nsite) continue;
     int x[4], st[4];
-    const int site = eo_site(g, h, 1, x, st);
+    int site = h;
+    if (FULL) site_coords(g, h, x, st);
+    else site = eo_site(g, h, 1, x, st);
     const bool clov = CL && g.clover;
     if (PREF && !clov) {
       own[threadIdx.x][0][0].fetch(in, a.Vmax, sa, h);
@@ -552,7 +555,7 @@ __global__ void __launch_bounds__(NT, MINB) k_eo2_odd(WArgs a, FieldPtr in, Fiel
     c2 acc[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k].re = acc[k].im = make_float2(0.f, 0.f);
-    eo_hop2<SPR, LPR>(g, mid, a.Vmax, sa, sb, site, x, st, bc2(mk2), acc);
+    eo_hop2<SPR, LPR, !FULL>(g, FULL ? in : mid, a.Vmax, sa, sb, site, x, st, bc2(mk2), acc);
     if (clov) {   // the 6x6 clover blocks need the whole spinor: lane by lane
 #pragma unroll
       for (int L = 0; L < 2; ++L) {

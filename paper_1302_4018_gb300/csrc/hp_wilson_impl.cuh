@@ -568,10 +568,85 @@ __global__ void __launch_bounds__(NT) k_bicg_xr(WArgs a) {
   }
 }
 
+enum { MASK_RUN = 0, MASK_GROUP = 1, MASK_EXACT = 2, MASK_FRESH = 3 };
+
+__device__ __forceinline__ bool eo_mask(const SlotState* S, int mask) {
+  if (mask == MASK_RUN) return S->status == SLOT_RUN;
+  if (mask == MASK_GROUP) return S->need_update == 1;
+  if (mask == MASK_FRESH) return S->status == SLOT_RUN && S->restart == 2 && S->need_update == 0;
+  return S->need_update == 2;
+}
+
+// The slots of an even-odd launch.  LOOP = false: one slot per block (grid x/z: the slot, y: the
+// tile), for launches that serve most slots; LOOP = true: a few blocks per tile (grid 1 x tiles x gz),
+// block z looping over the slots z, z + gz, ... that its mask selects, for launches that serve a few slots
+// at a time (the exact and group steps, fresh starts): an unselected slot then costs a flag, not a block.
+// The flags of up to NT slots are read at once, one per thread.  Every block reads a slot's mask before
+// that slot's finalisation (which waits for the last block that serves it, this one included), so the
+// blocks of a slot agree on it and the loop is uniform over the block.
+template <bool LOOP, int NT>
+struct EoSlots {
+  int p;   // the next candidate of this block's class (slot z + p gz): the only state kept over a slot's work
+  __device__ __forceinline__ EoSlots() : p(0) {}
+  __device__ __forceinline__ bool next(const SlotState* st, int mask, int nslots, int& slot) {
+    if constexpr (!LOOP) {
+      slot = (int)(blockIdx.z * gridDim.x + blockIdx.x);
+      return p++ == 0 && slot < nslots && eo_mask(st + slot, mask);
+    } else {
+      __shared__ unsigned int sel[NT / 32];
+      for (;;) {
+        if (p % NT == 0) {
+          const long long first = (long long)p * gridDim.z + blockIdx.z;
+          if (first >= nslots) return false;
+          const long long sl = first + (long long)threadIdx.x * gridDim.z;
+          const unsigned int b = __ballot_sync(0xffffffffu, sl < nslots && eo_mask(st + (sl < nslots ? sl : first), mask));
+          __syncthreads();   // the block is done with the flags before
+          if ((threadIdx.x & 31) == 0) sel[threadIdx.x >> 5] = b;
+          __syncthreads();
+        }
+        // every candidate of the chunk is looked at here, so p stops at a multiple of NT or behind a selected one
+        do {
+          const unsigned int rest = sel[(p % NT) >> 5] >> (p & 31);
+          if (rest) {
+            p += __ffs(rest);
+            slot = (p - 1) * (int)gridDim.z + (int)blockIdx.z;
+            return true;
+          }
+          p = (p | 31) + 1;
+        } while (p % NT);
+      }
+    }
+  }
+};
+
+#define EO_SLOTS_BEGIN(MASK, LOOP)                                                  \
+  EoSlots<(LOOP), NT> eo_slots_;                                                    \
+  for (int slot; eo_slots_.next(a.st, MASK, nslots, slot);) {                       \
+    SlotState* S = a.st + slot;                                                     \
+    const LatGeom g = a.lats[S->lat];                                               \
+    const int nsite = g.V >> 1;                                                     \
+    const int ntiles = (nsite + NT - 1) / NT;                                       \
+    if ((int)blockIdx.y >= ntiles) continue;                                        \
+    const int nparts = min((int)gridDim.y, ntiles);                                 \
+    double* part = a.part + (size_t)slot * 4 * a.gy;                                \
+    (void)nparts;                                                                   \
+    (void)part;
+#define EO_SLOTS_END }
+// the masked launches of the full-lattice iteration, in the same form
+#define FULL_SLOTS_BEGIN(MASK)                                                      \
+  EoSlots<true, NT> slots_;                                                         \
+  for (int slot; slots_.next(a.st, MASK, nslots, slot);) {                          \
+    SlotState* S = a.st + slot;                                                     \
+    const LatGeom g = a.lats[S->lat];                                               \
+    const int ntiles = (g.V + NT - 1) / NT;                                         \
+    if ((int)blockIdx.y >= ntiles) continue;                                        \
+    const int nparts = min((int)gridDim.y, ntiles);                                 \
+    double* part = a.part + (size_t)slot * 4 * a.gy;
+
 // ---- group update (FP32): r_g -= D e ; r = r_g ; (r^, r), ||r||^2   (x += e follows)
 template <int SPR, int EPR, int NT>
-__global__ void __launch_bounds__(NT) k_grp_update(WArgs a) {
-  SLOT_PREAMBLE(S->need_update == 1)
+__global__ void __launch_bounds__(NT) k_grp_update(WArgs a, int nslots) {
+  FULL_SLOTS_BEGIN(MASK_GROUP)
   typedef typename Real_of<SPR>::T R;
   float acc[3] = {0.f, 0.f, 0.f};
   for (int tile = blockIdx.y; tile < ntiles; tile += gridDim.y) {
@@ -613,6 +688,7 @@ __global__ void __launch_bounds__(NT) k_grp_update(WArgs a) {
       a.cnt[slot] = 0;
     }
   }
+  EO_SLOTS_END
 }
 
 // ---- reliable update, part 1: x += e ; e = 0
@@ -677,8 +753,8 @@ __device__ __forceinline__ void ru_finalize(WArgs& a, SlotState* S, const double
 // fixed-point links and solution, the hop in integer multiply-adds (48 bits: the
 // rounding error of b - D x is ~1e-14 ||b||, far below any tolerance the solver certifies).
 template <int SPR, int NT>
-__global__ void __launch_bounds__(NT, 3) k_ru_residual(WArgs a) {
-  SLOT_PREAMBLE(S->need_update == 2)
+__global__ void __launch_bounds__(NT, SPR == PR64 ? 3 : 2) k_ru_residual(WArgs a, int nslots) {
+  FULL_SLOTS_BEGIN(MASK_EXACT)
   typedef typename Real_of<SPR>::T R;
   const int comp = S->a, m = S->m;
   if (SPR == PR64) {
@@ -750,6 +826,7 @@ __global__ void __launch_bounds__(NT, 3) k_ru_residual(WArgs a) {
     block_sum_partials<3, NT>(part, a.gy, nparts, tot);
     if (threadIdx.x == 0) ru_finalize(a, S, tot, slot);
   }
+  EO_SLOTS_END
 }
 
 // ---- p = r + beta (p - omega v)   (restart: p = r^ = r)
@@ -860,15 +937,6 @@ static __global__ void k_w_grad(WArgs a, int lat, const int* __restrict__ slots,
 // is  r_o = b_o - d_o x_o + k H_oe x_e  while the even part vanishes by construction: the
 // certified residual is the residual of the full system.  Sites of one parity are numbered
 // by site >> 1 (every extent even: otherwise some hop joins sites of one parity and the split fails).
-enum { MASK_RUN = 0, MASK_GROUP = 1, MASK_EXACT = 2, MASK_FRESH = 3 };
-
-__device__ __forceinline__ bool eo_mask(const SlotState* S, int mask) {
-  if (mask == MASK_RUN) return S->status == SLOT_RUN;
-  if (mask == MASK_GROUP) return S->need_update == 1;
-  if (mask == MASK_FRESH) return S->status == SLOT_RUN && S->restart == 2 && S->need_update == 0;
-  return S->need_update == 2;
-}
-
 // full index and coordinates of half-site h of parity `par`
 __device__ __forceinline__ int eo_site(const LatGeom& g, int h, int par, int (&x)[4], int (&st)[4]) {
   const int l1h = g.L[0] >> 1;
@@ -934,62 +1002,6 @@ __device__ __forceinline__ void eo_hop(const LatGeom& g, FieldPtr in, int Vs, in
 
 __device__ __forceinline__ double leading_part(double v) { return v; }
 __device__ __forceinline__ double leading_part(ffl v) { return (double)v.hi; }
-
-// The slots of an even-odd launch.  LOOP = false: one slot per block (grid x/z: the slot, y: the
-// tile), for launches that serve most slots; LOOP = true: a few blocks per tile (grid 1 x tiles x gz),
-// block z looping over the slots z, z + gz, ... that its mask selects, for launches that serve a few slots
-// at a time (the exact and group steps, fresh starts): an unselected slot then costs a flag, not a block.
-// The flags of up to NT slots are read at once, one per thread.  Every block reads a slot's mask before
-// that slot's finalisation (which waits for the last block that serves it, this one included), so the
-// blocks of a slot agree on it and the loop is uniform over the block.
-template <bool LOOP, int NT>
-struct EoSlots {
-  int p;   // the next candidate of this block's class (slot z + p gz): the only state kept over a slot's work
-  __device__ __forceinline__ EoSlots() : p(0) {}
-  __device__ __forceinline__ bool next(const SlotState* st, int mask, int nslots, int& slot) {
-    if constexpr (!LOOP) {
-      slot = (int)(blockIdx.z * gridDim.x + blockIdx.x);
-      return p++ == 0 && slot < nslots && eo_mask(st + slot, mask);
-    } else {
-      __shared__ unsigned int sel[NT / 32];
-      for (;;) {
-        if (p % NT == 0) {
-          const long long first = (long long)p * gridDim.z + blockIdx.z;
-          if (first >= nslots) return false;
-          const long long sl = first + (long long)threadIdx.x * gridDim.z;
-          const unsigned int b = __ballot_sync(0xffffffffu, sl < nslots && eo_mask(st + (sl < nslots ? sl : first), mask));
-          __syncthreads();   // the block is done with the flags before
-          if ((threadIdx.x & 31) == 0) sel[threadIdx.x >> 5] = b;
-          __syncthreads();
-        }
-        // every candidate of the chunk is looked at here, so p stops at a multiple of NT or behind a selected one
-        do {
-          const unsigned int rest = sel[(p % NT) >> 5] >> (p & 31);
-          if (rest) {
-            p += __ffs(rest);
-            slot = (p - 1) * (int)gridDim.z + (int)blockIdx.z;
-            return true;
-          }
-          p = (p | 31) + 1;
-        } while (p % NT);
-      }
-    }
-  }
-};
-
-#define EO_SLOTS_BEGIN(MASK, LOOP)                                                  \
-  EoSlots<(LOOP), NT> eo_slots_;                                                    \
-  for (int slot; eo_slots_.next(a.st, MASK, nslots, slot);) {                       \
-    SlotState* S = a.st + slot;                                                     \
-    const LatGeom g = a.lats[S->lat];                                               \
-    const int nsite = g.V >> 1;                                                     \
-    const int ntiles = (nsite + NT - 1) / NT;                                       \
-    if ((int)blockIdx.y >= ntiles) continue;                                        \
-    const int nparts = min((int)gridDim.y, ntiles);                                 \
-    double* part = a.part + (size_t)slot * 4 * a.gy;                                \
-    (void)nparts;                                                                   \
-    (void)part;
-#define EO_SLOTS_END }
 
 // ---- even sites: mid = d_e^-1 hop(in_o)  (register caps: six resident blocks, <= 85 registers, for
 // the iteration's launches -- left alone the compiler takes 160 and halves the warps; four for the
@@ -1523,11 +1535,11 @@ struct WilsonEngine {
                        // 6 tensor-core even + pair odd (binary16, one lattice, no clover)
   int big_lat = 0;     // index of the largest lattice of the problem (set before setup)
   bool one_lat = false;   // the problem has one lattice (set before setup)
+  bool full2 = false;     // full-lattice iteration with two right-hand sides per thread
   int kernels_per_iteration() const { return eo ? (SPR == PR64 ? 10 : 12) : (SPR == PR64 ? 7 : 8); }
   // streaming kernels: grid-stride with 8 blocks per SM per slot (few partial sums and atomic tickets);
   // stencil kernels: one block per tile (gy) so that the lattice is swept once in site order
   dim3 grid() const { return dim3(nslots, gyb); }
-  dim3 grid_stencil() const { return dim3(nslots, gy); }
   // device memory of one slot's vectors (setup), for the scheduler's choice of the slot count
   static size_t slot_bytes(const WilsonEngine& e, int Vmax) {
     const size_t n = e.eo ? ((size_t)Vmax + 1) / 2 : (size_t)Vmax, S = SPR == PR64 ? 192 : SPR == PR32 ? 96 : 52;
@@ -1535,7 +1547,7 @@ struct WilsonEngine {
     return n * (7 * S + g + x + (e.eo ? x + S + g : 0));
   }
   // slots refilled together (the right-hand sides one thread carries must share a lattice)
-  int group() const { return (eo && SPR != PR64) ? 2 : rpt; }   // pairs also for eo_kernel 1 (any choice)
+  int group() const { return (full2 || (eo && SPR != PR64)) ? 2 : rpt; }   // pairs also for eo_kernel 1 (any choice)
 
   hp_status setup(int ns, int Vmax, const LatGeom* lats_dev, SlotState* st, const hp_solver_opts& o, double tol,
                   double delta, const LatGeom& gbig) {
@@ -1603,6 +1615,11 @@ struct WilsonEngine {
     } else if (eo) {
       // the full-lattice tuner cannot run on half-lattice fields: slot groups of 4 and 18-real links
       variant = 411;
+    } else if (SPR != PR64) {
+      // two right-hand sides per thread where their blocks (two tiles of a pair each) fill the GPU, else one per thread
+      // with 18-real links
+      full2 = (long long)((ns + 1) / 2) * ((gy + 1) / 2) >= 4LL * ctx->num_sms;
+      variant = 11;
     } else {
       k_w_fill<SPR><<<blocks_for(ctx, (long long)ns * Vmax, 256), 256, 0, ctx->stream>>>(a.p, Vmax, ns, 777ull);
       HP_LAUNCH_CHECK();
@@ -1860,7 +1877,31 @@ struct WilsonEngine {
     if (rpt == 2) return full ? stencil_steps_rpt<2, 18, CL>(which) : stencil_steps_rpt<2, 12, CL>(which);
     return full ? stencil_steps_rpt<1, 18, CL>(which) : stencil_steps_rpt<1, 12, CL>(which);
   }
-  hp_status stencil_step(int which) { return clover ? stencil_step_cl<true>(which) : stencil_step_cl<false>(which); }
+  // The V / T step of the full-lattice iteration with two right-hand sides per thread (hp_eo2.cuh), the form in FP32, FP16
+  // and BF16 where its blocks fill the GPU and the caller does not fix the other variants (rhs_per_thread), against the
+  // best of those: 24x15x27x19, two probes in FP16, 104 -> 92 ms a solve; 16^4, four probes, FP16 72.9 -> 64.0, clover
+  // FP32 117 -> 95; 15x10x12x18, two probes in BF16, 24.8 -> 24.2 (first call, without the variants' timing, 31.6 -> 25.9).
+  // On 5x6x7x4 with 48 slots its 96 blocks leave SMs idle: 6.4 against 5.1 ms.
+  template <bool CL>
+  hp_status full_pair(int which) {
+    if constexpr (SPR != PR64) {
+      constexpr int L16 = SPR == PR32 ? PR32 : PR16, TPB = 2;
+      const dim3 g2((nslots + 1) / 2, (gy + TPB - 1) / TPB, 1);
+      if (which == 0) {
+        ProfScope ps(ctx, SPR == PR32 ? "k_bicg_v<fp32>" : SPR == PR16 ? "k_bicg_v<fp16>" : "k_bicg_v<bf16>");
+        k_eo2_odd<SPR, L16, NT, 4, EPI_V, CL, TPB, true><<<g2, NT, 0, ctx->stream>>>(a, a.p, a.p, a.v, nslots);
+      } else {
+        ProfScope ps(ctx, SPR == PR32 ? "k_bicg_t<fp32>" : SPR == PR16 ? "k_bicg_t<fp16>" : "k_bicg_t<bf16>");
+        k_eo2_odd<SPR, L16, NT, 4, EPI_T, CL, TPB, true><<<g2, NT, 0, ctx->stream>>>(a, a.s, a.s, a.t, nslots);
+      }
+      HP_LAUNCH_CHECK();
+    }
+    return HP_OK;
+  }
+  hp_status stencil_step(int which) {
+    if (full2) return clover ? full_pair<true>(which) : full_pair<false>(which);
+    return clover ? stencil_step_cl<true>(which) : stencil_step_cl<false>(which);
+  }
   hp_status init() {
     if (eo) {
       {
@@ -1911,12 +1952,12 @@ struct WilsonEngine {
     { ProfScope ps(ctx, "k_bicg_xr"); k_bicg_xr<SPR, EPR, NT><<<grid(), NT, 0, ctx->stream>>>(a); }
     if (SPR != PR64) {
       ProfScope ps(ctx, "k_grp_update");
-      k_grp_update<SPR, EPR, NT><<<grid_stencil(), NT, 0, ctx->stream>>>(a);
+      k_grp_update<SPR, EPR, NT><<<tile_grid(), NT, 0, ctx->stream>>>(a, nslots);
     }
     { ProfScope ps(ctx, "k_ru_accum"); k_ru_accum<SPR, EPR, NT><<<grid(), NT, 0, ctx->stream>>>(a); }
     {
       ProfScope ps(ctx, SPR == PR64 ? "k_ru_residual<fp64>" : "k_ru_residual<ff>");
-      k_ru_residual<SPR, NT><<<grid_stencil(), NT, 0, ctx->stream>>>(a);
+      k_ru_residual<SPR, NT><<<tile_grid(), NT, 0, ctx->stream>>>(a, nslots);
     }
     { ProfScope ps(ctx, "k_bicg_p"); k_bicg_p<SPR, NT><<<grid(), NT, 0, ctx->stream>>>(a); }
     HP_LAUNCH_CHECK();

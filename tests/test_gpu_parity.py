@@ -740,6 +740,20 @@ def test_exact_residual_with_sites_of_different_magnitude(ctx, hp, dims, prec, e
         assert np.linalg.norm(r) <= (1e-10 + 1e-13) * np.linalg.norm(b)
 
 
+# the full-lattice steps with two right-hand sides per thread (enough slots to fill the GPU) and with one (fewer), against
+# the FP64 solver: every storage, the clover term, a pair with one slot left
+@pytest.mark.parametrize("prec,csw,block", [("fp32", 0.0, 108), ("fp16", 0.0, 108), ("bf16", 0.0, 107), ("fp16", 1.0, 108),
+                                            ("fp32", 1.0, 108), ("bf16", 0.0, 20)])
+def test_full_lattice_pair_kernels(ctx, hp, prec, csw, block):
+    dims, s = (9, 8, 7, 6), 9
+    U = synth.gauge_links(dims, 0.3, 55)
+    op = ctx.make_operator(hp.OP_WILSON, 0.02, 0.115, links_dev(U), dev(synth.mass_field(dims, 0.01, 3)), csw)
+    T, _, st = ctx.trace_inv(op, dims, s, 1e-10, ctx.make_opts(prec, rhs_block=block, z0_seed=5))
+    assert st["rhs_solved"] == 12 * s and st["max_true_residual"] <= 1e-10
+    T_ref, _, _ = ctx.trace_inv(op, dims, s, 1e-11, ctx.make_opts("fp64", z0_seed=5))
+    assert np.all(rel(T, T_ref) <= TRACE_RTOL)
+
+
 # ------------------------------------------------------------------ the comparison sequences (Section 5.2)
 @pytest.mark.parametrize("kind,dims,seed", [("natural", (8, 8, 8, 8), 0), ("natural", (2, 4, 8), 11),
                                             ("natural", (1024,), 3), ("z2", (4, 4, 4, 4), 12345),
