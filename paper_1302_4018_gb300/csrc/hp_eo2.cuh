@@ -526,7 +526,6 @@ __global__ void __launch_bounds__(NT, MINB) k_eo2_odd(WArgs a, FieldPtr in, Fiel
   const int ntiles = (nsite + NT - 1) / NT;
   const int nchunks = (ntiles + TPB - 1) / TPB;
   if ((int)blockIdx.y >= nchunks) return;
-  const int nparts = min((int)gridDim.y, nchunks);
   constexpr int NQ = EPI == EPI_V ? 2 : 3;
   constexpr int NF = 1;   // own-site field prefetched: the input (r^ of the V step is loaded after the hop)
   // (binary16 fields: 16 KB per field and block; the FP32 iteration's would exceed the 48 KB of
@@ -659,27 +658,4 @@ __global__ void __launch_bounds__(NT, MINB) k_eo2_odd(WArgs a, FieldPtr in, Fiel
     }
   }
   reduce_pair<NQ, NT>(dots, a.part + (size_t)sa * 4 * a.gy, a.part + (size_t)sb * 4 * a.gy, a.gy, two);
-#pragma unroll
-  for (int L = 0; L < 2; ++L) {
-    if (L == 1 && !two) break;
-    const int slot = L ? sb : sa;
-    SlotState* S = a.st + slot;
-    if (last_block(a.cnt + slot, nparts)) {
-      double tot[NQ];
-      block_sum_partials<NQ, NT>(a.part + (size_t)slot * 4 * a.gy, a.gy, nparts, tot);
-      if (threadIdx.x == 0) {
-        if (EPI == EPI_V) {
-          S->alpha = cdiv(S->rho, make_double2(tot[0], tot[1]));
-          S->restart = 0;
-          if (S->need_update == 3) S->need_update = 0;
-          S->sloppy_mv += 1;
-        } else {
-          S->omega = tot[NQ - 1] > 0.0 ? make_double2(tot[0] / tot[NQ - 1], tot[1] / tot[NQ - 1]) : make_double2(0.0, 0.0);
-          S->sloppy_mv += 1;
-        }
-        a.cnt[slot] = 0;
-      }
-      __syncthreads();
-    }
-  }
 }

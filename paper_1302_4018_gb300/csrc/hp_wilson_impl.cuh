@@ -477,6 +477,32 @@ __global__ void __launch_bounds__(NT) k_bicg_s(WArgs a) {
   }
 }
 
+// the scalar step of k_bicg_xr from its sums: beta, the breakdown test, the requests for updates (s: the state before)
+__device__ __forceinline__ void xr_step(const WArgs& a, SlotState* S, const SlotState& s, const double (&tot)[3]) {
+  const double2 rho_new = make_double2(tot[0], tot[1]);
+  const double rr = tot[2];
+  const bool bad = (s.omega.x == 0.0 && s.omega.y == 0.0) || (s.rho.x == 0.0 && s.rho.y == 0.0) ||
+                   (rho_new.x * rho_new.x + rho_new.y * rho_new.y) < 1e-28 * rr * s.rmax2 || !(rr == rr);
+  if (bad) {
+    S->restart = 1;               // r^ := r, p := r
+    S->rho = make_double2(rr, 0.0);
+    S->beta = make_double2(0.0, 0.0);
+  } else {
+    S->beta = dmul(cdiv(rho_new, s.rho), cdiv(s.alpha, s.omega));
+    S->rho = rho_new;
+  }
+  S->rnorm2 = rr;
+  S->iters = s.iters + 1;
+  if (s.iters + 1 >= a.maxiter) {
+    S->status = SLOT_FAIL;
+    S->need_update = 2;
+  } else if (rr <= a.tol2 * s.bnorm2 || rr < a.epsx2 * s.rexact2 || !(rr == rr)) {
+    S->need_update = 2;
+  } else if (rr < a.delta2 * s.rmax2) {
+    S->need_update = 1;
+  }
+}
+
 // ---- e += alpha p + omega s ; r = s - omega t ; rho' = (r^, r) ; ||r||^2
 template <int SPR, int EPR, int NT>
 __global__ void __launch_bounds__(NT) k_bicg_xr(WArgs a) {
@@ -536,36 +562,52 @@ __global__ void __launch_bounds__(NT) k_bicg_xr(WArgs a) {
     }
   }
   reduce_partials<R, 3, NT>(acc, part, a.gy);
-  if (last_block(a.cnt + slot, nparts)) {
+  if (SPR == PR64 && last_block(a.cnt + slot, nparts)) {   // FP64: the ticket hides behind the arithmetic; else k_xr_scalars
     double tot[3];
     block_sum_partials<3, NT>(part, a.gy, nparts, tot);
     if (threadIdx.x == 0) {
-      double2 rho_new = make_double2(tot[0], tot[1]);
-      double rr = tot[2];
-      double2 om2 = S->omega, rho = S->rho;
-      bool bad = (om2.x == 0.0 && om2.y == 0.0) || (rho.x == 0.0 && rho.y == 0.0) ||
-                 (rho_new.x * rho_new.x + rho_new.y * rho_new.y) < 1e-28 * rr * S->rmax2 || !(rr == rr);
-      if (bad) {
-        S->restart = 1;               // r^ := r, p := r
-        S->rho = make_double2(rr, 0.0);
-        S->beta = make_double2(0.0, 0.0);
-      } else {
-        S->beta = dmul(cdiv(rho_new, rho), cdiv(S->alpha, om2));
-        S->rho = rho_new;
-      }
-      S->rnorm2 = rr;
-      S->iters += 1;
-      if (S->iters >= a.maxiter) {
-        S->status = SLOT_FAIL;
-        S->need_update = 2;
-      } else if (rr <= a.tol2 * S->bnorm2 || rr < a.epsx2 * S->rexact2 || !(rr == rr)) {
-        S->need_update = 2;
-      } else if (rr < a.delta2 * S->rmax2) {
-        S->need_update = 1;
-      }
+      const SlotState s = *S;
+      xr_step(a, S, s, tot);
       a.cnt[slot] = 0;
     }
   }
+}
+
+// The partial sums of up to three quantities by one block of SCT threads, four warps per quantity; the sums in thread 0.
+// The scalar launches are pure latency (three of them an iteration), so everything that can be is loaded at once.
+constexpr int SCT = 384;
+__device__ __forceinline__ void scalar_sums(const double* part, int gy, int nparts, double (&tot)[3]) {
+  __shared__ double sh[SCT / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = w >> 2;
+  const double* p = part + (size_t)q * gy;
+  double t = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x & 127; i < nparts; i += 128) t += __ldcg(p + i);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  if (lane == 0) sh[w] = t;
+  __syncthreads();
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) tot[k] = (sh[4 * k] + sh[4 * k + 1]) + (sh[4 * k + 2] + sh[4 * k + 3]);
+}
+// the blocks of a slot: nparts of the caller where the problem has one lattice, else from the slot's lattice
+__device__ __forceinline__ int scalar_parts(const WArgs& a, const SlotState& S, int NT, int gym, int tpb, int one) {
+  if (one) return one;
+  const int V = a.lats[S.lat].V, nsite = a.eo ? V >> 1 : V;
+  return min(gym, ((nsite + NT - 1) / NT + tpb - 1) / tpb);
+}
+
+// the scalar step behind k_bicg_xr (grid height gym), one block per slot: beta, the breakdown test, the requests for updates
+template <int NT>
+__global__ void __launch_bounds__(SCT) k_xr_scalars(WArgs a, int gym, int one) {
+  SlotState* S = a.st + blockIdx.x;
+  const SlotState s = *S;
+  if (s.status != SLOT_RUN) return;
+  double tot[3];
+  scalar_sums(a.part + (size_t)blockIdx.x * 4 * a.gy, a.gy, scalar_parts(a, s, NT, gym, 1, one), tot);
+  if (threadIdx.x != 0) return;
+  xr_step(a, S, s, tot);
 }
 
 enum { MASK_RUN = 0, MASK_GROUP = 1, MASK_EXACT = 2, MASK_FRESH = 3 };
@@ -1036,6 +1078,33 @@ __global__ void __launch_bounds__(NT, SIN == PR64 ? 2 : (MASK == MASK_RUN ? 6 : 
   EO_SLOTS_END
 }
 
+__device__ __forceinline__ void vt_step(SlotState* S, const SlotState& s, int t_step, const double (&tot)[3]) {
+  if (t_step) {
+    S->omega = tot[2] > 0.0 ? make_double2(tot[0] / tot[2], tot[1] / tot[2]) : make_double2(0.0, 0.0);
+  } else {
+    S->alpha = cdiv(s.rho, make_double2(tot[0], tot[1]));
+    S->restart = 0;
+    if (s.need_update == 3) S->need_update = 0;
+  }
+  S->sloppy_mv = s.sloppy_mv + 1;
+}
+
+// The scalar step behind the V (alpha) and T (omega) kernels: one block per slot adds the partial sums of its blocks
+// (grid height `gym`, `tpb` tiles each).  A launch of its own, 3 us: with a ticket in the stencil kernels every one of
+// their blocks waits for its stores, a fence and an atomic before it leaves: 16^4, 96 slots, FP16, T step 225 -> 205 us, V
+// step 244 -> 217; 32^3x64 945 -> 850, 1003 -> 890.  (The FP64 solver keeps the ticket: its blocks are bound by the
+// FP64 pipe and hide it; 12^4 28.2 ms with it, 28.6 without.)
+template <int NT>
+__global__ void __launch_bounds__(SCT) k_step_scalars(WArgs a, int t_step, int gym, int tpb, int one) {
+  SlotState* S = a.st + blockIdx.x;
+  const SlotState s = *S;
+  if (s.status != SLOT_RUN) return;
+  double tot[3];   // V leaves the third quantity of an earlier kernel, unused
+  scalar_sums(a.part + (size_t)blockIdx.x * 4 * a.gy, a.gy, scalar_parts(a, s, NT, gym, tpb, one), tot);
+  if (threadIdx.x != 0) return;
+  vt_step(S, s, t_step, tot);
+}
+
 // ---- odd sites: out = d_o in - k^2 hop(mid), with the solver epilogues
 //   EPI_V: v = S p, (r^, v), alpha       EPI_T: t = S s, (t, s), (t, t), omega
 //   EPI_G: group update r_g -= S e, r = r_g, (r^, r_g), ||r_g||^2   (in = e, mid FP32)
@@ -1108,26 +1177,23 @@ __global__ void __launch_bounds__(NT, EO_ODD_MINB(SIN, REC)) k_eo_odd(WArgs a, F
     }
   }
   reduce_partials<R, NQ, NT>(dots, part, a.gy);
-  if (last_block(a.cnt + slot, nparts)) {
+  if ((EPI == EPI_G || SIN == PR64) && last_block(a.cnt + slot, nparts)) {   // V and T steps otherwise: k_step_scalars
     double tot[NQ];
     block_sum_partials<NQ, NT>(part, a.gy, nparts, tot);
-    if (threadIdx.x == 0) {
-      if (EPI == EPI_V) {
-        S->alpha = cdiv(S->rho, make_double2(tot[0], tot[1]));
-        S->restart = 0;
-        if (S->need_update == 3) S->need_update = 0;
-        S->sloppy_mv += 1;
-      } else if (EPI == EPI_T) {
-        S->omega = tot[NQ - 1] > 0.0 ? make_double2(tot[0] / tot[NQ - 1], tot[1] / tot[NQ - 1]) : make_double2(0.0, 0.0);
-        S->sloppy_mv += 1;
-      } else {
-        const double rr = tot[0];
-        S->rnorm2 = rr;
-        S->rmax2 = rr;
-        S->rho = S->restart ? make_double2(rr, 0.0) : make_double2(tot[1], tot[2]);
-        S->gupdates += 1;
-        S->need_update = (rr <= a.tol2 * S->bnorm2 || rr < a.epsx2 * S->rexact2) ? 2 : 3;
+    if (EPI != EPI_G) {
+      if (threadIdx.x == 0) {
+        const SlotState s = *S;
+        const double t3[3] = {tot[0], tot[1], tot[NQ - 1]};
+        vt_step(S, s, EPI == EPI_T, t3);
+        a.cnt[slot] = 0;
       }
+    } else if (threadIdx.x == 0) {
+      const double rr = tot[0];
+      S->rnorm2 = rr;
+      S->rmax2 = rr;
+      S->rho = S->restart ? make_double2(rr, 0.0) : make_double2(tot[1], tot[NQ - 1]);
+      S->gupdates += 1;
+      S->need_update = (rr <= a.tol2 * S->bnorm2 || rr < a.epsx2 * S->rexact2) ? 2 : 3;
       a.cnt[slot] = 0;
     }
   }
@@ -1536,7 +1602,7 @@ struct WilsonEngine {
   int big_lat = 0;     // index of the largest lattice of the problem (set before setup)
   bool one_lat = false;   // the problem has one lattice (set before setup)
   bool full2 = false;     // full-lattice iteration with two right-hand sides per thread
-  int kernels_per_iteration() const { return eo ? (SPR == PR64 ? 10 : 12) : (SPR == PR64 ? 7 : 8); }
+  int kernels_per_iteration() const { return eo ? (SPR == PR64 ? 10 : 15) : (SPR == PR64 ? 7 : full2 ? 11 : 9); }
   // streaming kernels: grid-stride with 8 blocks per SM per slot (few partial sums and atomic tickets);
   // stencil kernels: one block per tile (gy) so that the lattice is swept once in site order
   dim3 grid() const { return dim3(nslots, gyb); }
@@ -1648,6 +1714,14 @@ struct WilsonEngine {
   dim3 tile_grid() const {
     return dim3(1, gy, std::max(1, std::min({nslots, (ctx->num_sms * 16 + gy - 1) / gy, 64})));
   }
+  // partial sums per slot of a launch of height gym, tpb tiles per block, in a problem of one lattice
+  int parts(int gym, int tpb) const { return std::min(gym, ((a.Vmax + NT - 1) / NT + tpb - 1) / tpb); }
+  hp_status scalars(int which, int gym, int tpb) {
+    ProfScope ps(ctx, "k_step_scalars");
+    k_step_scalars<NT><<<nslots, SCT, 0, ctx->stream>>>(a, which, gym, tpb, one_lat ? parts(gym, tpb) : 0);
+    HP_LAUNCH_CHECK();
+    return HP_OK;
+  }
   template <int REC, bool CL>
   hp_status eo_schur(int which) {   // which: 0 v = S p, 1 t = S s, 2 group update with e
     dim3 gr = eo_grid();
@@ -1681,7 +1755,7 @@ struct WilsonEngine {
       k_eo_odd<EPR, PR32, PR32, 12, NT, EPI_G, CL><<<tile_grid(), NT, 0, ctx->stream>>>(a, a.e, a.mid32, a.rg, nslots);
     }
     HP_LAUNCH_CHECK();
-    return HP_OK;
+    return which < 2 && SPR != PR64 ? scalars(which, (int)gr.y, 1) : HP_OK;
   }
   // the V (which 0) or T (1) step with the pair kernels under a register budget of MINB blocks per SM,
   // links in LPR (binary16, or FP32: no conversions); the odd-site kernels sweep TPB tiles per block
@@ -1705,7 +1779,7 @@ struct WilsonEngine {
       k_eo2_odd<SPR, LPR, NT, MINB, EPI_T, CL, TPB><<<g2o, NT, 0, ctx->stream>>>(a, in, a.mid, out, nslots);
     }
     HP_LAUNCH_CHECK();
-    return HP_OK;
+    return scalars(which, (int)g2o.y, TPB);
   }
   // eo_kernel 5: the even-site pair kernel with the one-right-hand-side odd-site kernel
   template <bool CL>
@@ -1727,7 +1801,7 @@ struct WilsonEngine {
       k_eo_odd<SPR, SPR, LPR, 18, NT, EPI_T, CL><<<gr, NT, 0, ctx->stream>>>(a, in, a.mid, out, nslots);
     }
     HP_LAUNCH_CHECK();
-    return HP_OK;
+    return scalars(which, (int)gr.y, 1);
   }
   // the tensor-core even-site kernel serves binary16 iterations of one lattice without the clover
   // term, up to 32 slots (four MMA row groups)
@@ -1758,7 +1832,7 @@ struct WilsonEngine {
       k_eo2_odd<SPR, PR16, NT, 4, EPI_T, CL, TPB><<<g2o, NT, 0, ctx->stream>>>(a, in, a.mid, out, nslots);
     }
     HP_LAUNCH_CHECK();
-    return HP_OK;
+    return scalars(which, (int)g2o.y, TPB);
   }
   template <bool CL>
   hp_status eo_pair_v(int which) {   // eo_kernel = 10 L + B: B resident blocks, L = 1 FP32 links
@@ -1895,6 +1969,7 @@ struct WilsonEngine {
         k_eo2_odd<SPR, L16, NT, 4, EPI_T, CL, TPB, true><<<g2, NT, 0, ctx->stream>>>(a, a.s, a.s, a.t, nslots);
       }
       HP_LAUNCH_CHECK();
+      return scalars(which, (int)g2.y, TPB);
     }
     return HP_OK;
   }
@@ -1939,6 +2014,7 @@ struct WilsonEngine {
       { ProfScope ps(ctx, "k_bicg_s"); k_bicg_s<SPR, NT><<<grid(), NT, 0, ctx->stream>>>(a); }
       HP_TRY(eo_step(1));
       { ProfScope ps(ctx, "k_bicg_xr"); k_bicg_xr<SPR, EPR, NT><<<grid(), NT, 0, ctx->stream>>>(a); }
+      if (SPR != PR64) { ProfScope ps(ctx, "k_xr_scalars"); k_xr_scalars<NT><<<nslots, SCT, 0, ctx->stream>>>(a, gyb, one_lat ? parts(gyb, 1) : 0); }
       if (SPR != PR64) HP_TRY(eo_step(2));
       { ProfScope ps(ctx, "k_ru_accum"); k_ru_accum<SPR, EPR, NT><<<grid(), NT, 0, ctx->stream>>>(a); }
       HP_TRY(eo_exact());
@@ -1950,6 +2026,7 @@ struct WilsonEngine {
     { ProfScope ps(ctx, "k_bicg_s"); k_bicg_s<SPR, NT><<<grid(), NT, 0, ctx->stream>>>(a); }
     HP_TRY(stencil_step(1));
     { ProfScope ps(ctx, "k_bicg_xr"); k_bicg_xr<SPR, EPR, NT><<<grid(), NT, 0, ctx->stream>>>(a); }
+    if (SPR != PR64) { ProfScope ps(ctx, "k_xr_scalars"); k_xr_scalars<NT><<<nslots, SCT, 0, ctx->stream>>>(a, gyb, one_lat ? parts(gyb, 1) : 0); }
     if (SPR != PR64) {
       ProfScope ps(ctx, "k_grp_update");
       k_grp_update<SPR, EPR, NT><<<tile_grid(), NT, 0, ctx->stream>>>(a, nslots);
