@@ -1078,6 +1078,43 @@ __global__ void __launch_bounds__(NT, SIN == PR64 ? 2 : (MASK == MASK_RUN ? 6 : 
   EO_SLOTS_END
 }
 
+// the scalar step of a group update from its sums (||r_g||^2, (r^, r_g))
+__device__ __forceinline__ void grp_step(const WArgs& a, SlotState* S, const SlotState& s, const double (&tot)[3]) {
+  const double rr = tot[0];
+  S->rnorm2 = rr;
+  S->rmax2 = rr;
+  S->rho = s.restart ? make_double2(rr, 0.0) : make_double2(tot[1], tot[2]);
+  S->gupdates = s.gupdates + 1;
+  S->need_update = (rr <= a.tol2 * s.bnorm2 || rr < a.epsx2 * s.rexact2) ? 2 : 3;
+}
+// the scalar step of an exact residual: the start of a fresh slot, or the certified residual
+__device__ __forceinline__ void exact_step(WArgs& a, SlotState* S, const double (&tot)[3], int slot) {
+  if (S->restart == 2) {   // initial residual of the Schur system: start the iteration from it
+    S->restart = 0;
+    S->need_update = 0;
+    S->rnorm2 = S->rmax2 = S->rexact2 = tot[0];
+    S->rho = make_double2(tot[0], 0.0);
+    S->true_res2 = tot[0];
+    if (!(tot[0] > a.tol2 * S->bnorm2)) S->status = SLOT_DONE;
+    a.cnt[slot] = 0;
+  } else {
+    ru_finalize(a, S, tot, slot);
+  }
+}
+// the same behind the group (mask MASK_GROUP) and exact (MASK_EXACT) steps of the even-odd iteration in mixed precision
+// (32^3x64 per launch: group 302 -> 266 us, x_2 596 -> 546 us without their tickets)
+template <int NT>
+__global__ void __launch_bounds__(SCT) k_update_scalars(WArgs a, int mask, int gym, int one) {
+  SlotState* S = a.st + blockIdx.x;
+  if (!eo_mask(S, mask)) return;
+  const SlotState s = *S;
+  double tot[3];
+  scalar_sums(a.part + (size_t)blockIdx.x * 4 * a.gy, a.gy, scalar_parts(a, s, NT, gym, 1, one), tot);
+  if (threadIdx.x != 0) return;
+  if (mask == MASK_GROUP) grp_step(a, S, s, tot);
+  else exact_step(a, S, tot, blockIdx.x);
+}
+
 __device__ __forceinline__ void vt_step(SlotState* S, const SlotState& s, int t_step, const double (&tot)[3]) {
   if (t_step) {
     S->omega = tot[2] > 0.0 ? make_double2(tot[0] / tot[2], tot[1] / tot[2]) : make_double2(0.0, 0.0);
@@ -1177,23 +1214,13 @@ __global__ void __launch_bounds__(NT, EO_ODD_MINB(SIN, REC)) k_eo_odd(WArgs a, F
     }
   }
   reduce_partials<R, NQ, NT>(dots, part, a.gy);
-  if ((EPI == EPI_G || SIN == PR64) && last_block(a.cnt + slot, nparts)) {   // V and T steps otherwise: k_step_scalars
+  if (SIN == PR64 && last_block(a.cnt + slot, nparts)) {   // mixed: k_step_scalars, k_update_scalars
     double tot[NQ];
     block_sum_partials<NQ, NT>(part, a.gy, nparts, tot);
-    if (EPI != EPI_G) {
-      if (threadIdx.x == 0) {
-        const SlotState s = *S;
-        const double t3[3] = {tot[0], tot[1], tot[NQ - 1]};
-        vt_step(S, s, EPI == EPI_T, t3);
-        a.cnt[slot] = 0;
-      }
-    } else if (threadIdx.x == 0) {
-      const double rr = tot[0];
-      S->rnorm2 = rr;
-      S->rmax2 = rr;
-      S->rho = S->restart ? make_double2(rr, 0.0) : make_double2(tot[1], tot[NQ - 1]);
-      S->gupdates += 1;
-      S->need_update = (rr <= a.tol2 * S->bnorm2 || rr < a.epsx2 * S->rexact2) ? 2 : 3;
+    if (threadIdx.x == 0) {
+      const SlotState s = *S;
+      const double t3[3] = {tot[0], tot[1], tot[NQ - 1]};
+      vt_step(S, s, EPI == EPI_T, t3);
       a.cnt[slot] = 0;
     }
   }
@@ -1314,22 +1341,10 @@ __global__ void __launch_bounds__(NT, PX == PR64 ? EO_X_MINB : EO_X2_MINB) k_eo_
   }
   if (PX == PR64) reduce_partials<double, 3, NT>(accd, part, a.gy);
   else reduce_partials<float, 3, NT>(acc3, part, a.gy);
-  if (last_block(a.cnt + slot, nparts)) {
+  if (PX == PR64 && last_block(a.cnt + slot, nparts)) {   // mixed: k_update_scalars
     double tot[3];
     block_sum_partials<3, NT>(part, a.gy, nparts, tot);
-    if (threadIdx.x == 0) {
-      if (fresh) {   // initial residual of the Schur system: start the iteration from it
-        S->restart = 0;
-        S->need_update = 0;
-        S->rnorm2 = S->rmax2 = S->rexact2 = tot[0];
-        S->rho = make_double2(tot[0], 0.0);
-        S->true_res2 = tot[0];
-        if (!(tot[0] > a.tol2 * S->bnorm2)) S->status = SLOT_DONE;
-        a.cnt[slot] = 0;
-      } else {
-        ru_finalize(a, S, tot, slot);
-      }
-    }
+    if (threadIdx.x == 0) exact_step(a, S, tot, slot);
   }
   EO_SLOTS_END
 }
@@ -1602,7 +1617,7 @@ struct WilsonEngine {
   int big_lat = 0;     // index of the largest lattice of the problem (set before setup)
   bool one_lat = false;   // the problem has one lattice (set before setup)
   bool full2 = false;     // full-lattice iteration with two right-hand sides per thread
-  int kernels_per_iteration() const { return eo ? (SPR == PR64 ? 10 : 15) : (SPR == PR64 ? 7 : full2 ? 11 : 9); }
+  int kernels_per_iteration() const { return eo ? (SPR == PR64 ? 10 : 17) : (SPR == PR64 ? 7 : full2 ? 11 : 9); }
   // streaming kernels: grid-stride with 8 blocks per SM per slot (few partial sums and atomic tickets);
   // stencil kernels: one block per tile (gy) so that the lattice is swept once in site order
   dim3 grid() const { return dim3(nslots, gyb); }
@@ -1722,6 +1737,12 @@ struct WilsonEngine {
     HP_LAUNCH_CHECK();
     return HP_OK;
   }
+  hp_status update_scalars(int mask) {
+    ProfScope ps(ctx, "k_update_scalars");
+    k_update_scalars<NT><<<nslots, SCT, 0, ctx->stream>>>(a, mask, gy, one_lat ? parts(gy, 1) : 0);
+    HP_LAUNCH_CHECK();
+    return HP_OK;
+  }
   template <int REC, bool CL>
   hp_status eo_schur(int which) {   // which: 0 v = S p, 1 t = S s, 2 group update with e
     dim3 gr = eo_grid();
@@ -1755,7 +1776,8 @@ struct WilsonEngine {
       k_eo_odd<EPR, PR32, PR32, 12, NT, EPI_G, CL><<<tile_grid(), NT, 0, ctx->stream>>>(a, a.e, a.mid32, a.rg, nslots);
     }
     HP_LAUNCH_CHECK();
-    return which < 2 && SPR != PR64 ? scalars(which, (int)gr.y, 1) : HP_OK;
+    if (SPR == PR64) return HP_OK;
+    return which < 2 ? scalars(which, (int)gr.y, 1) : update_scalars(MASK_GROUP);
   }
   // the V (which 0) or T (1) step with the pair kernels under a register budget of MINB blocks per SM,
   // links in LPR (binary16, or FP32: no conversions); the odd-site kernels sweep TPB tiles per block
@@ -1929,7 +1951,7 @@ struct WilsonEngine {
       k_eo_x2<SPR, PX, NT><<<tile_grid(), NT, 0, ctx->stream>>>(a, nslots);
     }
     HP_LAUNCH_CHECK();
-    return HP_OK;
+    return SPR == PR64 ? HP_OK : update_scalars(MASK_EXACT);
   }
   template <int RPT, int REC, bool CL>
   hp_status stencil_steps_rpt(int which) {
