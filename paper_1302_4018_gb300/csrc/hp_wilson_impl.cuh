@@ -9,6 +9,7 @@
 #include <cstring>
 
 #include "hp_fields.cuh"
+#include "hp_reduce.cuh"
 
 static size_t field_bytes(int spr, int nslots, int Vmax, size_t* norm_bytes) {
   size_t per = spr == PR64 ? 192 : (spr == PR32 ? 96 : 48);
@@ -116,27 +117,6 @@ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
 }
 __device__ __forceinline__ double2 dmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-
-template <typename R, int NQ, int NT>
-__device__ __forceinline__ void reduce_partials(R (&v)[NQ], double* part, int gy) {
-  // warp level in the iteration precision, across warps in FP64
-  __shared__ double sh[NQ][NT / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    R t = v[q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) sh[q][warp] = (double)t;
-  }
-  __syncthreads();
-  if (threadIdx.x < NQ) {   // one thread per quantity: NT / 32 FP64 warp instructions a block, not NQ NT / 32
-    double t = 0.0;
-#pragma unroll
-    for (int w = 0; w < NT / 32; ++w) t += sh[threadIdx.x][w];
-    part[(size_t)threadIdx.x * gy + blockIdx.y] = t;
-  }
 }
 
 // diagonal 1 + m + mu(x) in the kernel's arithmetic (FP32 kernels read an FP32 copy of mu)
