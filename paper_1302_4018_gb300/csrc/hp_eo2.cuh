@@ -538,7 +538,9 @@ __global__ void __launch_bounds__(NT, MINB) k_eo2_odd(WArgs a, FieldPtr in, Fiel
 #pragma unroll
     for (int q = 0; q < NQ; ++q) dots[L][q] = 0.f;
   const float mk2 = FULL ? -(float)g.kappa : -(float)(g.kappa * g.kappa);
-  for (int tile = blockIdx.y * TPB; tile < min(ntiles, (int)(blockIdx.y + 1) * TPB); ++tile) {
+  // the chunks of TPB tiles blockIdx.y, blockIdx.y + gridDim.y, ...: one chunk, unless the lattice has more than the
+  // grid has rows
+  for (int tile = blockIdx.y * TPB; tile < ntiles; tile += (tile + 1) % TPB ? 1 : 1 + ((int)gridDim.y - 1) * TPB) {
     const int h = tile * NT + threadIdx.x;
     if (h >= nsite) continue;
     int x[4], st[4];

@@ -1,0 +1,47 @@
+"""Problems whose size passes a limit of the launches or of the memory."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1302_4018_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def hp():
+    from paper_1302_4018_gb300 import build as b
+
+    b.build()
+    from paper_1302_4018_gb300 import hprobe
+
+    return hprobe
+
+
+@pytest.fixture()
+def ctx(hp):   # a context of its own: the workspace goes with the test
+    torch.cuda.empty_cache()
+    c = hp.Context(0)
+    yield c
+    c.close()
+    torch.cuda.empty_cache()
+
+
+# More tiles of 128 sites than a grid has rows (65535), full lattice and even-odd pair kernels.  The links repeat those of a small
+# lattice and probe 0 is constant, so the solution repeats too: q per site and the iterations are those of the small
+# lattice (1e-9: both residuals are 1e-10, as in the parity tests).
+@pytest.mark.parametrize("dims,eo", [((64, 64, 64, 34), 0), ((64, 64, 64, 66), 1)])
+def test_wilson_lattice_of_more_tiles_than_grid_rows(ctx, hp, dims, eo):
+    small = (8, 8, 8, 2)
+    U = synth.gauge_links(small, 0.3, 61)
+    u = torch.from_numpy(U.view(np.float64).reshape(*small[::-1], 72)).to("cuda:0")
+    opts = dict(z0_seed=0, even_odd=eo, rhs_block=4, eo_kernel=4)
+    ref, _, st0 = ctx.trace_inv(ctx.make_operator(hp.OP_WILSON, 0.05, 0.11, u.reshape(-1)), small, 1, 1e-10,
+                                ctx.make_opts("fp64", **opts))
+    big = u.repeat(*(a // b for a, b in zip(dims[::-1], small[::-1])), 1).reshape(-1)
+    T, _, st = ctx.trace_inv(ctx.make_operator(hp.OP_WILSON, 0.05, 0.11, big), dims, 1, 1e-10,
+                             ctx.make_opts("fp16", maxiter=2 * st0["iterations_max"] + 20, **opts))
+    assert st["max_true_residual"] <= 1e-10
+    scale = np.prod(dims) / np.prod(small)
+    assert np.all(np.abs(T - scale * ref) <= 1e-9 * np.abs(T))
