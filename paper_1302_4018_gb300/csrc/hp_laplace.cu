@@ -1226,7 +1226,7 @@ __device__ __forceinline__ double cluster_sum(ClusterSum<CLT>& cs, double v, int
 }
 
 template <bool MF, int CLT>
-__device__ __forceinline__ void cg_cluster_solve(const LArgs& a, const LatGeom& g, SlotState& S, ClusterSum<CLT>& cs, int item,
+__device__ __forceinline__ void cg_cluster_solve(const LArgs& a, const LatGeom& g, SlotState& S, ClusterSum<CLT>& cs, int cid,
                                                  double* x, double* r, double* p, double* q, int C, int rank, int most) {
   const int lo = (int)((long long)g.V * rank / C), hi = (int)((long long)g.V * (rank + 1) / C);
   const int m = S.m, pa = S.a;
@@ -1235,7 +1235,7 @@ __device__ __forceinline__ void cg_cluster_solve(const LArgs& a, const LatGeom& 
   double acc = 0.0, tot;
   if (S.status == SLOT_INIT) {
     for (int i = lo + threadIdx.x; i < hi; i += CLT) {
-      const double b = lap_src(g, a, item, i, m, pa);
+      const double b = lap_src(g, a, cid, i, m, pa);
       x[i] = 0.0;
       r[i] = b;
       p[i] = b;
@@ -1282,7 +1282,7 @@ __device__ __forceinline__ void cg_cluster_solve(const LArgs& a, const LatGeom& 
     if (S.need_update) {   // the true residual r = b - A x
       acc = 0.0;
       for (int i = lo + threadIdx.x; i < hi; i += CLT) {
-        const double rv = lap_src(g, a, item, i, m, pa) - lap_site<MF, false>(g, diag0, x, i);
+        const double rv = lap_src(g, a, cid, i, m, pa) - lap_site<MF, false>(g, diag0, x, i);
         r[i] = rv;
         acc = fma(rv, rv, acc);
       }
@@ -1302,12 +1302,13 @@ __device__ __forceinline__ void cg_cluster_solve(const LArgs& a, const LatGeom& 
   }
   if (S.status == SLOT_RUN) return;
   acc = 0.0;
-  for (int i = lo + threadIdx.x; i < hi; i += CLT) acc = fma(lap_src(g, a, item, i, m, pa), x[i], acc);
+  for (int i = lo + threadIdx.x; i < hi; i += CLT) acc = fma(lap_src(g, a, cid, i, m, pa), x[i], acc);
   tot = cluster_sum(cs, acc, C, rank, gen);   // no block leaves before the others have written their sums to it
   if (threadIdx.x == 0) S.q = make_double2(tot, 0.0);
 }
 
-// item = first + number of the cluster; the vectors of an item of the launch at its number times Vmax.  (Vectors in
+// item = first + number of the cluster; the vectors of an item of the launch at its number times Vmax, its deflation
+// coefficients at its number times defl_k.  (Vectors in
 // shared memory, one block of 131 KB per SM, measured slower than two blocks with the vectors in L2: 8^4, 256 vectors 1.66
 // against 1.47 ms.)
 template <int CLT>
@@ -1321,16 +1322,16 @@ __global__ void __launch_bounds__(CLT, 1024 / CLT) k_cg_cluster(LArgs a, int fir
   const LatGeom g = a.lats[S.lat];
   const size_t off = (size_t)cid * a.Vmax;
   if (C > 1) cluster_barrier(C);   // every block of the cluster has started: its shared memory can be written
-  if (g.mass_field) cg_cluster_solve<true, CLT>(a, g, S, cs, item, a.x + off, a.r + off, a.p + off, a.q + off, C, rank, most);
-  else cg_cluster_solve<false, CLT>(a, g, S, cs, item, a.x + off, a.r + off, a.p + off, a.q + off, C, rank, most);
+  if (g.mass_field) cg_cluster_solve<true, CLT>(a, g, S, cs, cid, a.x + off, a.r + off, a.p + off, a.q + off, C, rank, most);
+  else cg_cluster_solve<false, CLT>(a, g, S, cs, cid, a.x + off, a.r + off, a.p + off, a.q + off, C, rank, most);
   __syncthreads();
   if (threadIdx.x == 0 && rank == 0) a.st[item] = S;
 }
 
-// How a problem of n right-hand sides of V sites (on average) runs: C blocks of `threads` per right-hand side; C = 0: the
-// slot engine.
+// How a problem of n right-hand sides of V sites (on average) runs: C blocks of `threads` per right-hand side, `wave`
+// right-hand sides per launch; C = 0: the slot engine.
 struct ClusterPlan {
-  int C, threads;
+  int C, threads, wave;
   int most;   // iterations per launch: about a second's worth at the most (a solve that needs more is launched again)
 };
 // The cost of an iteration over all right-hand sides in SM cycles: FP64 (6.5 cycles a site at 2 lanes per clock, at 0.8 of
@@ -1339,25 +1340,47 @@ struct ClusterPlan {
 // launches.  At equal cost the larger cluster: two blocks of 512 threads share an SM and fill each other's waits; blocks
 // that are alone on theirs take 1024 threads.  Both sides measured (clusters / slots): 64^3 with 32 vectors 24.0 / 30.8
 // ms, 16 23.4 / 15.0, 64 58.5 / 60; 32^3 with 2 1.9 / 2.8, 64 5.6 / 8.0; 8^4 with 1 0.51 / 1.1, 64 0.55 / 1.75.
-static ClusterPlan cluster_plan(const hp_ctx* ctx, double n, double V) {
-  ClusterPlan pl = {0, 512, 0};
+// Clusters of several blocks stop where they lose: 80^3 with 38 vectors 41.5 / 47.8 ms, 152 138 / 176; 96^3 with 38 95.6 /
+// 76.5, 152 361 / 284; 128^3 with 38 184 / 175.  One block per right-hand side still wins there (96^3 with 304 vectors
+// 402 / 564 ms), as far as the vectors of the resident blocks (two per SM) find room.
+// Room: 1 GB, else a 32nd of the device's memory (9.3 GB) and half of what is free or held for them already; the workspace
+// stays with the context.
+constexpr double CLUSTER_MAX_SITES = 600e3;   // of a cluster of several blocks
+static hp_status cluster_plan(const hp_ctx* ctx, double n, double V, int Vmax, ClusterPlan* out) {
+  ClusterPlan pl = {0, 512, 0, 0};
+  const double per = 32.0 * Vmax, gb = (double)(1 << 30);   // four vectors
+  double room = -1.0;
   double best = 1.4 * n * V * 6.5 / ctx->num_sms + 60e3;
   for (int C = 1; C <= 8; C *= 2) {
-    if (C > 1 && V < 1024.0 * C) break;
+    if (C > 1 && (V < 1024.0 * C || V > CLUSTER_MAX_SITES)) break;
     const double k = std::ceil(n * C / ctx->num_sms);   // blocks on the busiest SM
     const double cost = (k == 1.0 && V / C > 8192.0 ? 1.9 : 1.25 * k) * V * 6.5 / C + (C == 1 ? 5e3 : 18e3);
-    if (cost <= best) {
-      best = cost;
-      pl.C = C;
-      pl.threads = k == 1.0 ? 1024 : 512;
+    if (!(cost <= best)) continue;
+    const double resident = std::min(n, std::max(1.0, (double)(2 * ctx->num_sms / C)));
+    if (per * resident > gb) {
+      if (room < 0.0) {
+        size_t free_b = 0, total_b = 0, held = 0;
+        HP_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        for (const char* name : {"solve.lx", "solve.lr", "solve.lp", "solve.lq"}) {
+          auto it = ctx->ws.find(name);
+          if (it != ctx->ws.end()) held += it->second.bytes;
+        }
+        room = std::min(total_b / 32.0, (free_b + held) / 2.0);
+      }
+      if (per * resident > room) continue;
     }
+    best = cost;
+    pl.C = C;
+    pl.threads = k == 1.0 ? 1024 : 512;
+    pl.wave = (int)std::min(n, std::max(resident, std::floor(gb / per)));
   }
   pl.most = (int)std::max(16.0, std::min(1024.0, 2e9 / best));
-  return pl;
+  *out = pl;
+  return HP_OK;
 }
 
 static hp_status solve_laplace_clusters(hp_ctx* ctx, SolveProblem& pb, SolveResult& res, const ClusterPlan& pl) {
-  const int C = pl.C, most = pl.most;
+  const int C = pl.C, most = pl.most, wave = pl.wave;
   const auto t0 = std::chrono::steady_clock::now();
   const int nl = (int)pb.lats.size();
   int Vmax = 0;
@@ -1382,9 +1405,6 @@ static hp_status solve_laplace_clusters(hp_ctx* ctx, SolveProblem& pb, SolveResu
       }
   }
   const int n = (int)items.size();
-  // right-hand sides per launch: as many as are resident at once, up to 1 GB of vectors beyond that
-  const int resident = std::max(1, 2 * ctx->num_sms / C);
-  const int wave = (int)std::min<long long>(n, std::max<long long>(resident, (1LL << 30) / (32LL * Vmax)));
   LArgs a;
   memset(&a, 0, sizeof(a));
   void* p = nullptr;
@@ -1406,17 +1426,8 @@ static hp_status solve_laplace_clusters(hp_ctx* ctx, SolveProblem& pb, SolveResu
   }
   const int defl_k = pb.lats[0].defl_k;
   if (defl_k) {
-    HP_TRY(hp_ws(ctx, "solve.defl_c", sizeof(double) * (size_t)n * defl_k, &p));
+    HP_TRY(hp_ws(ctx, "solve.defl_c", sizeof(double) * (size_t)wave * defl_k, &p));
     a.dc = (double*)p;
-    const int rows = 32768;   // grid limit of one dimension
-    for (int i0 = 0; i0 < n; i0 += rows) {
-      LArgs b = a;
-      b.st += i0;
-      b.dc += (size_t)i0 * defl_k;
-      ProfScope ps(ctx, "k_cg_defl");
-      k_cg_defl<256><<<dim3(defl_k, std::min(rows, n - i0)), 256, 0, ctx->stream>>>(b);
-    }
-    HP_LAUNCH_CHECK();
   }
   int* dev_slots = nullptr;
   std::vector<int> ident;
@@ -1429,6 +1440,17 @@ static hp_status solve_laplace_clusters(hp_ctx* ctx, SolveProblem& pb, SolveResu
   void (*kern)(LArgs, int, int, int) = pl.threads == 1024 ? k_cg_cluster<1024> : k_cg_cluster<512>;
   for (int i0 = 0; i0 < n; i0 += wave) {
     const int nw = std::min(wave, n - i0);
+    if (defl_k) {
+      const int rows = 32768;   // grid limit of one dimension
+      for (int j0 = 0; j0 < nw; j0 += rows) {
+        LArgs b = a;
+        b.st += i0 + j0;
+        b.dc += (size_t)j0 * defl_k;
+        ProfScope ps(ctx, "k_cg_defl");
+        k_cg_defl<256><<<dim3(defl_k, std::min(rows, nw - j0)), 256, 0, ctx->stream>>>(b);
+      }
+      HP_LAUNCH_CHECK();
+    }
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)(nw * C));
@@ -1501,13 +1523,19 @@ hp_status hp_solve_laplace(hp_ctx* ctx, SolveProblem& pb, SolveResult& res) {
   // the caller who fixes the slots, the chunk or the graph replay gets the slot engine
   if (pb.opts.rhs_block <= 0 && pb.opts.check_every <= 0 && !pb.opts.use_graph) {
     double n = 0.0, work = 0.0;
+    int Vmax = 1;
     for (size_t L = 0; L < pb.lats.size(); ++L) {
+      Vmax = std::max(Vmax, pb.lats[L].V);
       const double k = (double)(pb.s_max[L] - pb.first[L]) * pb.lats[L].parts;
       n += k;
       work += k * pb.lats[L].V;
     }
-    const ClusterPlan pl = cluster_plan(ctx, n, work / n);
-    if (pl.C && n <= 1e6) return solve_laplace_clusters(ctx, pb, res, pl);
+    ClusterPlan pl;
+    HP_TRY(cluster_plan(ctx, n, work / n, Vmax, &pl));
+    if (pl.C && n <= 1e6) {
+      const hp_status st = solve_laplace_clusters(ctx, pb, res, pl);
+      if (st != HP_ENOMEM) return st;   // no room for them (seen before the first launch): the slot engine takes less
+    }
   }
   LaplaceEngine e{ctx};
   return run_schedule(ctx, e, pb, res, 12, 0.0);

@@ -45,3 +45,22 @@ def test_wilson_lattice_of_more_tiles_than_grid_rows(ctx, hp, dims, eo):
     assert st["max_true_residual"] <= 1e-10
     scale = np.prod(dims) / np.prod(small)
     assert np.all(np.abs(T - scale * ref) <= 1e-9 * np.abs(T))
+
+
+# A solve per cluster keeps every resident right-hand side's vectors: 304 of 128^3 would hold 20 GB where the slot engine
+# takes 0.8, and 76 of 64^3 find no room (0.64 GB) on a device with 0.4 GB left, where the slot engine (0.13) still does.
+# 1e-7: q = z^T x to |r| / lambda_min with residuals of 1e-9 |b|, against the slot engine with its own.
+@pytest.mark.parametrize("dims,s,leave,most", [((128, 128, 128), 304, None, 9.4e9), ((64, 64, 64), 76, 0.4e9, 0.4e9)])
+def test_laplacian_workspace_is_bounded(ctx, hp, dims, s, leave, most):
+    op = ctx.make_operator(hp.OP_LAPLACIAN, 0.3)
+    opts = dict(z0_seed=4, probe_kind="z2")
+    ref, _, _ = ctx.trace_inv(op, dims, 2, 1e-9, ctx.make_opts("fp64", rhs_block=2, **opts))
+    free = torch.cuda.mem_get_info()[0]
+    filler = None if leave is None else torch.empty(int(free - leave), dtype=torch.uint8, device="cuda:0")
+    before = torch.cuda.mem_get_info()[0]
+    T, _, st = ctx.trace_inv(op, dims, s, 1e-9, ctx.make_opts("fp64", **opts))
+    used = before - torch.cuda.mem_get_info()[0]
+    del filler
+    assert st["rhs_solved"] == s and st["max_true_residual"] <= 1e-9
+    assert used <= most
+    assert np.all(np.abs(T[:2] - ref) <= 1e-7 * np.abs(ref))
