@@ -1343,6 +1343,9 @@ struct ClusterPlan {
 // Clusters of several blocks stop where they lose: 80^3 with 38 vectors 41.5 / 47.8 ms, 152 138 / 176; 96^3 with 38 95.6 /
 // 76.5, 152 361 / 284; 128^3 with 38 184 / 175.  One block per right-hand side still wins there (96^3 with 304 vectors
 // 402 / 564 ms), as far as the vectors of the resident blocks (two per SM) find room.
+// A batch of uneven lattices takes at least as long as one solve of its largest on one cluster, against the slot engine's
+// rounds of launches: 256 vectors of 8^4 with two of 64^3 took 53.7 ms with one block per right-hand side, 15.5 with four
+// (slots 27); 64 of 8^4 with one of 64^3 13.7, slots 9.8.
 // Room: 1 GB, else a 32nd of the device's memory (9.3 GB) and half of what is free or held for them already; the workspace
 // stays with the context.
 constexpr double CLUSTER_MAX_SITES = 600e3;   // of a cluster of several blocks
@@ -1350,11 +1353,14 @@ static hp_status cluster_plan(const hp_ctx* ctx, double n, double V, int Vmax, C
   ClusterPlan pl = {0, 512, 0, 0};
   const double per = 32.0 * Vmax, gb = (double)(1 << 30);   // four vectors
   double room = -1.0;
-  double best = 1.4 * n * V * 6.5 / ctx->num_sms + 60e3;
+  const double slots = std::max(12.0, std::min(256.0, std::floor((double)(4 << 20) / Vmax)));
+  const double rounds = Vmax > V ? std::ceil(n / slots) : 1.0;
+  double best = 1.4 * n * V * 6.5 / ctx->num_sms + 60e3 * rounds;
   for (int C = 1; C <= 8; C *= 2) {
-    if (C > 1 && (V < 1024.0 * C || V > CLUSTER_MAX_SITES)) break;
+    if (C > 1 && (V < 1024.0 * C || Vmax > CLUSTER_MAX_SITES)) break;
     const double k = std::ceil(n * C / ctx->num_sms);   // blocks on the busiest SM
-    const double cost = (k == 1.0 && V / C > 8192.0 ? 1.9 : 1.25 * k) * V * 6.5 / C + (C == 1 ? 5e3 : 18e3);
+    const double alone = (Vmax / C > 8192.0 ? 1.9 : 1.25) * Vmax * 6.5 / C;
+    const double cost = std::max(1.25 * k * V * 6.5 / C, alone) + (C == 1 ? 5e3 : 18e3);
     if (!(cost <= best)) continue;
     const double resident = std::min(n, std::max(1.0, (double)(2 * ctx->num_sms / C)));
     if (per * resident > gb) {

@@ -64,3 +64,21 @@ def test_laplacian_workspace_is_bounded(ctx, hp, dims, s, leave, most):
     assert st["rhs_solved"] == s and st["max_true_residual"] <= 1e-9
     assert used <= most
     assert np.all(np.abs(T[:2] - ref) <= 1e-7 * np.abs(ref))
+
+
+# The Laplacian's route for a batch: a solve per cluster (a few launches) where the lattices are alike, but not where one
+# solve of the largest on one block outlasts all the others (the slot engine launches four kernels an iteration).
+@pytest.mark.parametrize("batch,clusters", [([((8, 8, 8, 8), 64), ((64, 64, 64), 1)], False),
+                                            ([((8, 8, 8, 8), 64), ((16, 16, 16), 64)], True),
+                                            ([((12, 12, 12), 20), ((16, 16, 16), 20), ((24, 24, 24), 20)], True)])
+def test_laplacian_batch_route_and_values(ctx, hp, batch, clusters):
+    dims, s = zip(*batch)
+    ops = [ctx.make_operator(hp.OP_LAPLACIAN, 0.3)] * len(batch)
+    opts = dict(z0_seed=4, probe_kind="z2")
+    n0 = ctx.launch_count()
+    T, st = ctx.trace_inv_batch(ops, dims, s, 1e-10, ctx.make_opts("fp64", **opts))
+    launches = ctx.launch_count() - n0
+    assert st["max_true_residual"] <= 1e-10 and (launches < 4 * st["iterations_max"]) == clusters
+    ref, _ = ctx.trace_inv_batch(ops, dims, s, 1e-10, ctx.make_opts("fp64", rhs_block=16, **opts))
+    for a, b in zip(T, ref):
+        assert np.all(np.abs(a - b) <= 1e-8 * np.abs(b))
