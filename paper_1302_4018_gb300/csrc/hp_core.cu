@@ -113,6 +113,16 @@ hp_status hp_ws(hp_ctx* ctx, const char* name, size_t bytes, void** out) {
   return HP_OK;
 }
 
+hp_status hp_ws_release(hp_ctx* ctx, const char* prefix) {
+  HP_CUDA(cudaStreamSynchronize(ctx->stream));
+  for (auto& kv : ctx->ws)
+    if (kv.first.compare(0, strlen(prefix), prefix) == 0 && kv.second.p) {
+      HP_CUDA(cudaFree(kv.second.p));
+      kv.second = DevBuf();
+    }
+  return HP_OK;
+}
+
 hp_status hp_ws_free_all(hp_ctx* ctx) {
   for (auto& kv : ctx->ws)
     if (kv.second.p) cudaFree(kv.second.p);

@@ -171,6 +171,8 @@ struct hp_ctx {
 
 // workspace
 hp_status hp_ws(hp_ctx* ctx, const char* name, size_t bytes, void** out);
+// gives back the buffers whose names begin with prefix (what a setup took before it found no room for the rest)
+hp_status hp_ws_release(hp_ctx* ctx, const char* prefix);
 hp_status hp_ws_free_all(hp_ctx* ctx);
 
 // profiling around a launch

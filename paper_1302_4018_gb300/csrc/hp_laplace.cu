@@ -1515,16 +1515,17 @@ hp_status hp_solve_laplace(hp_ctx* ctx, SolveProblem& pb, SolveResult& res) {
     // in a block of 128; FP64 64 ms, 95)
     const long long nq = (long long)(pb.s_max[0] - pb.first[0]) * pb.lats[0].parts;
     const bool mixed = pb.opts.precision == HP_PREC_MIXED_FP32;
-    const int want = pb.opts.rhs_block > 0 ? pb.opts.rhs_block : nq <= 32 ? 32 : (mixed && nq > 96 ? 128 : 64);
-    pb.opts.rhs_block = want <= 32 ? 32 : (want <= 64 ? 64 : 128);
-    if (mixed) {
-      if (want <= 32) return run_blocked<1, true>(ctx, pb, res);
-      if (want <= 64) return run_blocked<2, true>(ctx, pb, res);
-      return run_blocked<4, true>(ctx, pb, res);
-    }
-    if (want <= 32) return run_blocked<1, false>(ctx, pb, res);
-    if (want <= 64) return run_blocked<2, false>(ctx, pb, res);
-    return run_blocked<4, false>(ctx, pb, res);
+    const bool automatic = pb.opts.rhs_block <= 0;
+    const int want = automatic ? (nq <= 32 ? 32 : (mixed && nq > 96 ? 128 : 64)) : pb.opts.rhs_block;
+    auto run = [&](int B) {
+      pb.opts.rhs_block = B;
+      if (mixed) return B == 32 ? run_blocked<1, true>(ctx, pb, res) : B == 64 ? run_blocked<2, true>(ctx, pb, res) : run_blocked<4, true>(ctx, pb, res);
+      return B == 32 ? run_blocked<1, false>(ctx, pb, res) : B == 64 ? run_blocked<2, false>(ctx, pb, res) : run_blocked<4, false>(ctx, pb, res);
+    };
+    const hp_status st = run(want <= 32 ? 32 : (want <= 64 ? 64 : 128));
+    if (st != HP_ENOMEM || !automatic || want <= 64) return st;
+    HP_TRY(hp_ws_release(ctx, "solve."));   // a wide block that found no room (before its first launch)
+    return run(64);
   }
   // the caller who fixes the slots, the chunk or the graph replay gets the slot engine
   if (pb.opts.rhs_block <= 0 && pb.opts.check_every <= 0 && !pb.opts.use_graph) {
@@ -1540,7 +1541,8 @@ hp_status hp_solve_laplace(hp_ctx* ctx, SolveProblem& pb, SolveResult& res) {
     HP_TRY(cluster_plan(ctx, n, work / n, Vmax, &pl));
     if (pl.C && n <= 1e6) {
       const hp_status st = solve_laplace_clusters(ctx, pb, res, pl);
-      if (st != HP_ENOMEM) return st;   // no room for them (seen before the first launch): the slot engine takes less
+      if (st != HP_ENOMEM) return st;
+      HP_TRY(hp_ws_release(ctx, "solve."));   // no room for them (seen before the first launch): the slot engine takes less
     }
   }
   LaplaceEngine e{ctx};

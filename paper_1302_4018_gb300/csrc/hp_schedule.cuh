@@ -86,14 +86,21 @@ hp_status run_schedule(hp_ctx* ctx, Engine& eng, SolveProblem& pb, SolveResult& 
   for (int L = 1; L < nl; ++L)
     if (pb.lats[L].V > pb.lats[big].V) big = L;
 
-  void* p = nullptr;
-  HP_TRY(hp_ws(ctx, "solve.lats", sizeof(LatGeom) * nl, &p));
-  LatGeom* lats_dev = (LatGeom*)p;
-  HP_CUDA(cudaMemcpyAsync(lats_dev, pb.lats.data(), sizeof(LatGeom) * nl, cudaMemcpyHostToDevice, ctx->stream));
-  HP_TRY(hp_ws(ctx, "solve.state", sizeof(SlotState) * nslots, &p));
-  SlotState* st_dev = (SlotState*)p;
-  HP_TRY(hp_ws(ctx, "solve.slots", sizeof(int) * nslots, &p));
-  int* dev_slots = (int*)p;
+  LatGeom* lats_dev = nullptr;
+  SlotState* st_dev = nullptr;
+  int* dev_slots = nullptr;
+  auto buffers = [&]() -> hp_status {
+    void* p = nullptr;
+    HP_TRY(hp_ws(ctx, "solve.lats", sizeof(LatGeom) * nl, &p));
+    lats_dev = (LatGeom*)p;
+    HP_CUDA(cudaMemcpyAsync(lats_dev, pb.lats.data(), sizeof(LatGeom) * nl, cudaMemcpyHostToDevice, ctx->stream));
+    HP_TRY(hp_ws(ctx, "solve.state", sizeof(SlotState) * nslots, &p));
+    st_dev = (SlotState*)p;
+    HP_TRY(hp_ws(ctx, "solve.slots", sizeof(int) * nslots, &p));
+    dev_slots = (int*)p;
+    return HP_OK;
+  };
+  HP_TRY(buffers());
   std::vector<SlotState> host(nslots);
   memset(host.data(), 0, sizeof(SlotState) * nslots);
   eng.big_lat = big;
@@ -102,6 +109,8 @@ hp_status run_schedule(hp_ctx* ctx, Engine& eng, SolveProblem& pb, SolveResult& 
   if (su == HP_ENOMEM && automatic && nslots > small_slots) {   // fragmented memory: the smaller slot count
     nslots = (small_slots + Engine::GROUP_MAX - 1) / Engine::GROUP_MAX * Engine::GROUP_MAX;
     host.resize(nslots);
+    HP_TRY(hp_ws_release(ctx, "solve."));
+    HP_TRY(buffers());
     su = eng.setup(nslots, Vmax, lats_dev, st_dev, pb.opts, pb.tol, delta, pb.lats[big]);
   }
   HP_TRY(su);

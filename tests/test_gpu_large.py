@@ -82,3 +82,18 @@ def test_laplacian_batch_route_and_values(ctx, hp, batch, clusters):
     ref, _ = ctx.trace_inv_batch(ops, dims, s, 1e-10, ctx.make_opts("fp64", rhs_block=16, **opts))
     for a, b in zip(T, ref):
         assert np.all(np.abs(a - b) <= 1e-8 * np.abs(b))
+
+
+# More than 96 right-hand sides in FP32 run in a block of 128 (1.6 GB here) where that finds room, else in the block of
+# 64 (0.8 GB) they always had.  Both blocks iterate to 1e-9 |b|; 1e-7 as above.
+def test_sparse_block_width_falls_back_to_the_room_there_is(ctx):
+    rp, ci, val = synth.grid_matrix((80, 80, 80), 5, shift=0.3)
+    rp, ci, val = (torch.from_numpy(np.ascontiguousarray(a)).to("cuda:0") for a in (rp, ci, val))
+    paths = torch.zeros((1, 80 ** 3), dtype=torch.int32, device="cuda:0")
+    opts = dict(z0_seed=4, probe_kind="z2")
+    ref, _, _ = ctx.trace_inv_sparse(rp, ci, val, paths, [1], 2, 1e-9, ctx.make_opts("fp32", rhs_block=32, **opts))
+    filler = torch.empty(int(torch.cuda.mem_get_info()[0] - 0.7e9), dtype=torch.uint8, device="cuda:0")
+    T, _, st = ctx.trace_inv_sparse(rp, ci, val, paths, [1], 100, 1e-9, ctx.make_opts("fp32", **opts))
+    del filler
+    assert st["rhs_solved"] == 100 and st["max_true_residual"] <= 1e-9
+    assert np.all(np.abs(T[:2] - ref) <= 1e-7 * np.abs(ref))
