@@ -233,7 +233,8 @@ hp_status hp_trace_inv(hp_ctx* ctx, const hp_operator* op, const hp_lattice* lat
  * right-hand sides it solves (Wilson only): right-hand side j = 12 (m - first) + a
  * of x_out (device, complex128 [n_keep][V][4][3] in the canonical layout of
  * hp_operator_apply) receives the converged A^-1 v_{m,a} as the solver holds it
- * (FP64, or the float-float solution of the mixed modes rounded to FP64).
+ * (FP64, or the block fixed-point solution of the mixed modes, 2^-51 of the
+ * site's largest component, rounded to FP64).
  * With them a caller checks ||v_{m,a} - A x_{m,a}|| / ||v_{m,a}|| and
  * q_m = sum_a v_{m,a}^H x_{m,a} independently of the library (Section 1.1.2:
  * each quadrature is a linear solve).  n_keep = 0 is hp_trace_inv.

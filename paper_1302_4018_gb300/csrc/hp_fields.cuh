@@ -20,6 +20,7 @@
 // (the 18-real forms trade bytes, shared by all right-hand sides of a launch,
 // for the reconstruction arithmetic of the ALU-bound sloppy stencil)
 #pragma once
+#include "hp_fixed.cuh"
 #include "hp_internal.h"
 
 // ----------------------------------------------------------------- float-float
@@ -67,7 +68,6 @@ __device__ __forceinline__ ffl& operator-=(ffl& a, ffl b) {
   a = a - b;
   return a;
 }
-__device__ __forceinline__ double ffl_to_double(ffl a) { return (double)a.hi + (double)a.lo; }
 template <typename T>
 struct is_ffl {
   static constexpr bool value = false;
@@ -182,15 +182,12 @@ struct SpinorIO<PR32> {
   }
 };
 
-// Block fixed point, the storage of the float-float solutions: component = (i + l) unit with a 28-bit integer i, an FP32
-// remainder l (|l| < 5) and a power of two `unit` per site (nrm), such that |i| <= 2^27: 49 bits below the site's
-// largest component.  p: int4 [6], lo: float4 [6], in the chunks of SpinorIO<PR32>.  The integers are what the exact hop
-// multiplies (hop_ff).  A component that is not finite makes the unit NaN, and the site with it.
-__device__ __forceinline__ ffl fix_value(int i, float l, float unit) {
-  const float f = (float)(i >> 4) * 16.0f, b = (float)(i & 15) + l;   // both conversions exact
-  const float s = __fadd_rn(f, b), bb = __fsub_rn(s, f);
-  const float e = __fadd_rn(__fsub_rn(f, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-  return ffl(s * unit, e * unit);
+// Block fixed point (hp_fixed.cuh): p: int4 [6], lo: float4 [6], in the chunks of SpinorIO<PR32>, nrm: the units.  The
+// integers are what the exact hop multiplies (hop_ff).  A component that is not finite makes the unit NaN, and the site with it.
+__device__ __forceinline__ ffl fix_ffl(int i, float l, float unit) {
+  ffl v;
+  fix_value(i, l, unit, v.hi, v.lo);
+  return v;
 }
 
 template <>
@@ -211,8 +208,8 @@ struct SpinorIO<PRFF> {
     }
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      s[2 * k] = {R(fix_value(h[k].x, l[k].x, u)), R(fix_value(h[k].y, l[k].y, u))};
-      s[2 * k + 1] = {R(fix_value(h[k].z, l[k].z, u)), R(fix_value(h[k].w, l[k].w, u))};
+      s[2 * k] = {R(fix_ffl(h[k].x, l[k].x, u)), R(fix_ffl(h[k].y, l[k].y, u))};
+      s[2 * k + 1] = {R(fix_ffl(h[k].z, l[k].z, u)), R(fix_ffl(h[k].w, l[k].w, u))};
     }
   }
   template <typename R>
@@ -228,9 +225,8 @@ struct SpinorIO<PRFF> {
       finite = finite && a < INFINITY && b < INFINITY;
       m = fmaxf(m, fmaxf(a, b));
     }
-    // m < 2^(E - 126) with E its biased exponent; unit = 2^(E - 126 - 27)
-    const int E = max(__float_as_int(m) >> 23, 37);
-    const float unit = __int_as_float((E - 26) << 23), inv = __int_as_float((280 - E) << 23);
+    float unit, inv;
+    fix_unit(m, unit, inv);
     int4* p = (int4*)f.p + (size_t)slot * 6 * Vmax + site;
     float4* q = (float4*)f.lo + (size_t)slot * 6 * Vmax + site;
 #pragma unroll
@@ -239,11 +235,7 @@ struct SpinorIO<PRFF> {
       int i[4];
       float l[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float t = v[j].hi * inv;   // exact; an integer already where it has no room for a fraction
-        i[j] = __float2int_rn(t);
-        l[j] = fmaf(v[j].lo, inv, t - (float)i[j]);
-      }
+      for (int j = 0; j < 4; ++j) fix_split(v[j].hi, v[j].lo, inv, i[j], l[j]);
       p[(size_t)k * Vmax] = make_int4(i[0], i[1], i[2], i[3]);
       q[(size_t)k * Vmax] = make_float4(l[0], l[1], l[2], l[3]);
     }
@@ -260,15 +252,14 @@ struct SpinorIO<PRFF> {
     }
     f.nrm[(size_t)slot * Vmax + site] = 0.f;
   }
-  // one component
+  // one component in FP64, as stored: what the certified residual belongs to
   __device__ static __forceinline__ double2 component(FieldPtr f, int Vmax, int slot, int site, int comp) {
     const size_t off = ((size_t)slot * 6 + comp / 2) * Vmax + site;
     const int4 h = ((const int4*)f.p)[off];
     const float4 l = ((const float4*)f.lo)[off];
     const float u = f.nrm[(size_t)slot * Vmax + site];
-    const ffl a = (comp & 1) ? fix_value(h.z, l.z, u) : fix_value(h.x, l.x, u);
-    const ffl b = (comp & 1) ? fix_value(h.w, l.w, u) : fix_value(h.y, l.y, u);
-    return make_double2(ffl_to_double(a), ffl_to_double(b));
+    return (comp & 1) ? make_double2(((double)h.z + (double)l.z) * u, ((double)h.w + (double)l.w) * u)
+                      : make_double2(((double)h.x + (double)l.x) * u, ((double)h.y + (double)l.y) * u);
   }
 };
 
@@ -759,7 +750,7 @@ __device__ __forceinline__ void hop_ff(const LatGeom& g, FieldPtr in, int Vmax, 
         }
     }
     const int sh = min(63, (__float_as_int(umax) - __float_as_int(un[hn])) >> 23);
-    const float sc = __int_as_float((127 - sh) << 23);
+    const float sc = __int_as_float((97 - sh) << 23);   // 2^(-30 - sh)
     cplx<long long> w[6];
     cplx<float> wl[6];
 #pragma unroll
@@ -794,12 +785,12 @@ __device__ __forceinline__ void hop_ff(const LatGeom& g, FieldPtr in, int Vmax, 
       default: accumulate<3, 1>(acc, w); accumulate<3, 1>(accl, wl); break;
     }
   }
-  // (acc + accl) 2^-30 umax: 24 leading bits, the 24 below them, and the rest with the cross terms
-  const float scale = umax * 0x1p-30f + 0.0f * usum;
+  // (acc 2^-30 + accl) umax: 24 leading bits, the 24 below them, and the rest with the cross terms
+  const float scale = umax + 0.0f * usum;
   auto value = [scale](long long a, float l) {
-    const float top = (float)(int)(a >> 39) * 0x1p39f;
+    const float top = (float)(int)(a >> 39) * 0x1p9f;
     const long long rest = a & 0x7fffffffffLL;
-    const float low = fmaf((float)(int)(rest >> 15), 0x1p15f, (float)(int)(rest & 0x7fff) + l);
+    const float low = fmaf((float)(int)(rest >> 15), 0x1p-15f, fmaf((float)(int)(rest & 0x7fff), 0x1p-30f, l));
     const float s = __fadd_rn(top, low), bb = __fsub_rn(s, top);
     const float e = __fadd_rn(__fsub_rn(top, __fsub_rn(s, bb)), __fsub_rn(low, bb));
     return ffl(s * scale, e * scale);
