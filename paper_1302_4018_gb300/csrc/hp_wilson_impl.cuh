@@ -491,7 +491,8 @@ __global__ void __launch_bounds__(NT) k_bicg_xr(WArgs a) {
   typedef R RE;
   static_assert(SPR == EPR, "the solution increment is kept in the iteration precision");
   // plain chains of FMAs: two per complex multiply-add and real part, where a product subtracted from a product costs a
-  // third operation (FP64 vectors are bound by the FP64 pipe: 12^4, 12 slots, xr 85 -> 58, p 45 -> 30, s 28 -> 18 us)
+  // third operation (FP64 vectors are bound by the FP64 pipe: 12^4, 12 slots, xr 85 -> 63, p 45 -> 30, s 28 -> 18 us).
+  // e sums many small increments, so each is formed first and added once: one rounding at e's magnitude, not four.
   const R ax = (R)S->alpha.x, ay = (R)S->alpha.y, ox = (R)S->omega.x, oy = (R)S->omega.y;
   R acc[3] = {0, 0, 0};
   for (int tile = blockIdx.y; tile < ntiles; tile += gridDim.y) {
@@ -505,8 +506,8 @@ __global__ void __launch_bounds__(NT) k_bicg_xr(WArgs a) {
       for (int k = 0; k < 12; ++k) {
         const size_t o = (size_t)k * a.Vmax;
         const double2 p = __ldg(pp + o), sv = __ldg(ps + o), t = __ldg(pt + o), h = __ldg(ph + o), e = pe[o];
-        pe[o] = make_double2(fma(ax, p.x, fma(-ay, p.y, fma(ox, sv.x, fma(-oy, sv.y, e.x)))),
-                             fma(ax, p.y, fma(ay, p.x, fma(ox, sv.y, fma(oy, sv.x, e.y)))));
+        pe[o] = make_double2(e.x + fma(ax, p.x, fma(-ay, p.y, fma(ox, sv.x, -oy * sv.y))),
+                             e.y + fma(ax, p.y, fma(ay, p.x, fma(ox, sv.y, oy * sv.x))));
         const double rx = fma(oy, t.y, fma(-ox, t.x, sv.x)), ry = fma(-oy, t.x, fma(-ox, t.y, sv.y));
         pr[o] = make_double2(rx, ry);
         acc[0] = fma(h.x, rx, fma(h.y, ry, acc[0]));
@@ -525,8 +526,8 @@ __global__ void __launch_bounds__(NT) k_bicg_xr(WArgs a) {
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
       const RE px = (RE)p[k].x, py = (RE)p[k].y, sx = (RE)s[k].x, sy = (RE)s[k].y;
-      e[k].x = fma(ax, px, fma(-ay, py, fma(ox, sx, fma(-oy, sy, e[k].x))));
-      e[k].y = fma(ax, py, fma(ay, px, fma(ox, sy, fma(oy, sx, e[k].y))));
+      e[k].x += fma(ax, px, fma(-ay, py, fma(ox, sx, -oy * sy)));
+      e[k].y += fma(ax, py, fma(ay, px, fma(ox, sy, oy * sx)));
       s[k].x = fma(oy, t[k].y, fma(-ox, t[k].x, s[k].x));
       s[k].y = fma(-oy, t[k].x, fma(-ox, t[k].y, s[k].y));
     }
