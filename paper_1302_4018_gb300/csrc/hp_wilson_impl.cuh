@@ -1679,9 +1679,10 @@ struct WilsonEngine {
       variant = 411;
     } else if (SPR != PR64) {
       // two right-hand sides per thread where their blocks (two tiles of a pair each) fill the GPU, else one per thread
-      // with 18-real links
+      // with 12-real links in FP32 (12^4 in 4, 8, 12 slots: 12.0, 10.2, 7.8 ms a solve, 18-real 13.4, 11.1, 8.3) and 18-real
+      // links in FP16 and BF16 (16^3x8 in 4 slots FP16 15.5 ms, 12-real 16.0)
       full2 = (long long)((ns + 1) / 2) * ((gy + 1) / 2) >= 4LL * ctx->num_sms;
-      variant = 11;
+      variant = SPR == PR32 ? 10 : 11;
     } else {
       k_w_fill<SPR><<<blocks_for(ctx, (long long)ns * Vmax, 256), 256, 0, ctx->stream>>>(a.p, Vmax, ns, 777ull);
       HP_LAUNCH_CHECK();
