@@ -474,8 +474,8 @@ struct LaplaceEngine {
   bool one_lat = false;   // one lattice in the problem (set by the scheduler; unused here)
   int defl_k = 0;
   dim3 grid() const { return dim3(nslots, gy); }
-  // keeps the scheduler at 4M sites' worth of slots: 128^2x64 with 32 vectors took 116 ms in 12 slots, 122 in 32
-  static size_t slot_bytes(const LaplaceEngine&, int) { return (size_t)8 << 30; }
+  // 4M sites' worth of slots: 128^2x64 with 32 vectors took 116 ms in 12 slots, 122 in 32
+  static constexpr bool MORE_SLOTS = false;
   int group() const { return 1; }
   hp_status setup(int ns, int Vmax, const LatGeom* lats_dev, SlotState* st, const hp_solver_opts& o, double tol,
                   double, const LatGeom& big) {
@@ -1064,7 +1064,7 @@ struct BlockedSparseEngine {
   long long nnz = 0;
   double delta = 0.0;
   int group() const { return 1; }
-  static size_t slot_bytes(const BlockedSparseEngine&, int Vmax) { return 32 * (size_t)Vmax; }   // rhs_block is always set
+  static constexpr bool MORE_SLOTS = false;   // rhs_block is always set
   hp_status setup(int ns, int Vmax, const LatGeom* lats_dev, SlotState* st, const hp_solver_opts& o, double tol,
                   double, const LatGeom&) {
     if (ns != B) {

@@ -66,15 +66,17 @@ hp_status run_schedule(hp_ctx* ctx, Engine& eng, SolveProblem& pb, SolveResult& 
   const int small_slots = (int)std::max(12LL, std::min((4LL << 20) / std::max(1, Vmax), 256LL));
   if (automatic) {
     nslots = small_slots;
-    const size_t per = Engine::slot_bytes(eng, Vmax);
-    const long long fit = (long long)((8ULL << 30) / std::max<size_t>(1, per));
-    long long want = std::min<long long>({(long long)queue.size(), 256LL, fit});
-    if (want > nslots) {
-      size_t free_b = 0, total_b = 0, held = 0;
-      HP_CUDA(cudaMemGetInfo(&free_b, &total_b));
-      for (auto& kv : ctx->ws)
-        if (kv.first.compare(0, 6, "solve.") == 0) held += kv.second.bytes;
-      if (per * (size_t)want <= (free_b + held) / 2) nslots = (int)want;
+    if constexpr (Engine::MORE_SLOTS) {
+      const size_t per = Engine::slot_bytes(eng, Vmax);
+      const long long fit = (long long)((8ULL << 30) / std::max<size_t>(1, per));
+      const long long want = std::min<long long>({(long long)queue.size(), 256LL, fit});
+      if (want > nslots) {
+        size_t free_b = 0, total_b = 0, held = 0;
+        HP_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        for (auto& kv : ctx->ws)
+          if (kv.first.compare(0, 6, "solve.") == 0) held += kv.second.bytes;
+        if (per * (size_t)want <= (free_b + held) / 2) nslots = (int)want;
+      }
     }
     const long long rounds = ((long long)queue.size() + nslots - 1) / nslots;
     if (rounds > 1 && nslots > small_slots) nslots = (int)(((long long)queue.size() + rounds - 1) / rounds);

@@ -74,8 +74,8 @@ static int dslash_gridy(hp_ctx* ctx, int V, int NT, int nslots) {
 //                  solve stops when this true residual is <= tol ||b||.
 // FP64 solves run the same iteration in FP64 with exact updates only.
 // All scalars live per slot in device memory; reductions are deterministic
-// (fixed shuffle trees, per-block partials summed in block order by the
-// block that finishes last).
+// (fixed shuffle trees, per-block partials summed in a fixed order by the
+// block that finishes last, or by a small launch in the mixed precisions).
 struct WArgs {
   const LatGeom* lats;
   SlotState* st;
@@ -119,6 +119,28 @@ __device__ __forceinline__ double2 dmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
+// the scalar step of V (alpha) or T (omega) from its sums ((r^, v), or (t, s) and (t, t) third; s: the state before)
+__device__ __forceinline__ void vt_step(SlotState* S, const SlotState& s, int t_step, const double (&tot)[3]) {
+  if (t_step) {
+    S->omega = tot[2] > 0.0 ? make_double2(tot[0] / tot[2], tot[1] / tot[2]) : make_double2(0.0, 0.0);
+  } else {
+    S->alpha = cdiv(s.rho, make_double2(tot[0], tot[1]));
+    S->restart = 0;
+    if (s.need_update == 3) S->need_update = 0;
+  }
+  S->sloppy_mv = s.sloppy_mv + 1;
+}
+
+// the scalar step of a group update from its sums (||r_g||^2, (r^, r_g))
+__device__ __forceinline__ void grp_step(const WArgs& a, SlotState* S, const SlotState& s, const double (&tot)[3]) {
+  const double rr = tot[0];
+  S->rnorm2 = rr;
+  S->rmax2 = rr;
+  S->rho = s.restart ? make_double2(rr, 0.0) : make_double2(tot[1], tot[2]);
+  S->gupdates = s.gupdates + 1;
+  // 3: group update done, x += e pending (k_ru_accum); cleared by the next V step
+  S->need_update = (rr <= a.tol2 * s.bnorm2 || rr < a.epsx2 * s.rexact2) ? 2 : 3;
+}
 // diagonal 1 + m + mu(x) in the kernel's arithmetic (FP32 kernels read an FP32 copy of mu)
 template <typename R>
 __device__ __forceinline__ R site_diag(const LatGeom& g, int site) {
@@ -333,14 +355,9 @@ __global__ void __launch_bounds__(NT) k_wds(WArgs a, FieldPtr in, FieldPtr out, 
     block_sum_partials<NQ, NT>(a.part + (size_t)(slot0 + r) * 4 * a.gy, a.gy, nparts, tot);
     if (threadIdx.x == 0) {
       SlotState* S = a.st + slot0 + r;
-      if (EPI == EPI_V) {
-        S->alpha = cdiv(S->rho, make_double2(tot[0], tot[1]));
-        S->restart = 0;
-        if (S->need_update == 3) S->need_update = 0;
-      } else {
-        S->omega = tot[NQ - 1] > 0.0 ? make_double2(tot[0] / tot[NQ - 1], tot[1] / tot[NQ - 1]) : make_double2(0.0, 0.0);
-      }
-      S->sloppy_mv += 1;
+      const SlotState s = *S;
+      const double t3[3] = {tot[0], tot[1], tot[NQ - 1]};
+      vt_step(S, s, EPI == EPI_T, t3);
       a.cnt[slot0 + r] = 0;
     }
   }
@@ -605,7 +622,7 @@ __device__ __forceinline__ bool eo_mask(const SlotState* S, int mask) {
 // block z looping over the slots z, z + gz, ... that its mask selects, for launches that serve a few slots
 // at a time (the exact and group steps, fresh starts): an unselected slot then costs a flag, not a block.
 // The flags of up to NT slots are read at once, one per thread.  Every block reads a slot's mask before
-// that slot's finalisation (which waits for the last block that serves it, this one included), so the
+// that slot's finalisation (by the last block that serves it, this one included, or by a later launch), so the
 // blocks of a slot agree on it and the loop is uniform over the block.
 template <bool LOOP, int NT>
 struct EoSlots {
@@ -701,13 +718,8 @@ __global__ void __launch_bounds__(NT) k_grp_update(WArgs a, int nslots) {
     double tot[3];
     block_sum_partials<3, NT>(part, a.gy, nparts, tot);
     if (threadIdx.x == 0) {
-      const double rr = tot[0];
-      S->rnorm2 = rr;
-      S->rmax2 = rr;
-      S->rho = S->restart ? make_double2(rr, 0.0) : make_double2(tot[1], tot[2]);
-      S->gupdates += 1;
-      // 3: group update done, x += e pending (k_ru_accum); cleared by the next k_bicg_v
-      S->need_update = (rr <= a.tol2 * S->bnorm2 || rr < a.epsx2 * S->rexact2) ? 2 : 3;
+      const SlotState s = *S;
+      grp_step(a, S, s, tot);
       a.cnt[slot] = 0;
     }
   }
@@ -1059,15 +1071,6 @@ __global__ void __launch_bounds__(NT, SIN == PR64 ? 2 : (MASK == MASK_RUN ? 6 : 
   EO_SLOTS_END
 }
 
-// the scalar step of a group update from its sums (||r_g||^2, (r^, r_g))
-__device__ __forceinline__ void grp_step(const WArgs& a, SlotState* S, const SlotState& s, const double (&tot)[3]) {
-  const double rr = tot[0];
-  S->rnorm2 = rr;
-  S->rmax2 = rr;
-  S->rho = s.restart ? make_double2(rr, 0.0) : make_double2(tot[1], tot[2]);
-  S->gupdates = s.gupdates + 1;
-  S->need_update = (rr <= a.tol2 * s.bnorm2 || rr < a.epsx2 * s.rexact2) ? 2 : 3;
-}
 // the scalar step of an exact residual: the start of a fresh slot, or the certified residual
 __device__ __forceinline__ void exact_step(WArgs& a, SlotState* S, const double (&tot)[3], int slot) {
   if (S->restart == 2) {   // initial residual of the Schur system: start the iteration from it
@@ -1094,17 +1097,6 @@ __global__ void __launch_bounds__(SCT) k_update_scalars(WArgs a, int mask, int g
   if (threadIdx.x != 0) return;
   if (mask == MASK_GROUP) grp_step(a, S, s, tot);
   else exact_step(a, S, tot, blockIdx.x);
-}
-
-__device__ __forceinline__ void vt_step(SlotState* S, const SlotState& s, int t_step, const double (&tot)[3]) {
-  if (t_step) {
-    S->omega = tot[2] > 0.0 ? make_double2(tot[0] / tot[2], tot[1] / tot[2]) : make_double2(0.0, 0.0);
-  } else {
-    S->alpha = cdiv(s.rho, make_double2(tot[0], tot[1]));
-    S->restart = 0;
-    if (s.need_update == 3) S->need_update = 0;
-  }
-  S->sloppy_mv = s.sloppy_mv + 1;
 }
 
 // The scalar step behind the V (alpha) and T (omega) kernels: one block per slot adds the partial sums of its blocks
@@ -1602,7 +1594,8 @@ struct WilsonEngine {
   // streaming kernels: grid-stride with 8 blocks per SM per slot (few partial sums and atomic tickets);
   // stencil kernels: one block per tile (gy) so that the lattice is swept once in site order
   dim3 grid() const { return dim3(nslots, gyb); }
-  // device memory of one slot's vectors (setup), for the scheduler's choice of the slot count
+  static constexpr bool MORE_SLOTS = true;   // more slots than 4M sites' worth pay (the scheduler's choice)
+  // device memory of one slot's vectors (setup)
   static size_t slot_bytes(const WilsonEngine& e, int Vmax) {
     const size_t n = e.eo ? ((size_t)Vmax + 1) / 2 : (size_t)Vmax, S = SPR == PR64 ? 192 : SPR == PR32 ? 96 : 52;
     const size_t x = 192, g = SPR == PR64 ? 0 : 96;   // solution (one parity), FP32 group residual / intermediate
@@ -1667,9 +1660,8 @@ struct WilsonEngine {
     a.delta2 = delta * delta;
     a.epsx2 = SPR == PR64 ? 0.0 : 1e-10;   // FP64 true residual after a 1e5 reduction
     a.maxiter = o.maxiter > 0 ? o.maxiter : 10000;
-    // right-hand sides per thread of the stencil: fixed by the caller or autotuned on the largest lattice
-    // stencil variant: fixed by the caller (right-hand sides per thread, 12-real links) or autotuned
-    // on the largest lattice of the problem
+    // stencil variant: fixed by the caller (right-hand sides per thread, link form), else by rule, or timed on the largest
+    // lattice of the problem (FP64, full lattice)
     const int forced = o.rhs_per_thread % 100, full = (o.rhs_per_thread / 100) % 10 == 1,
               group = o.rhs_per_thread / 1000;
     if (forced == 1 || forced == 2 || forced == 4) {
@@ -1677,7 +1669,7 @@ struct WilsonEngine {
     } else if (eo) {
       // the full-lattice tuner cannot run on half-lattice fields: slot groups of 4 and 18-real links
       variant = 411;
-    } else if (SPR != PR64) {
+    } else if constexpr (SPR != PR64) {
       // two right-hand sides per thread where their blocks (two tiles of a pair each) fill the GPU, else one per thread
       // with 12-real links in FP32 (12^4 in 4, 8, 12 slots: 12.0, 10.2, 7.8 ms a solve, 18-real 13.4, 11.1, 8.3) and 18-real
       // links in FP16 and BF16 (16^3x8 in 4 slots FP16 15.5 ms, 12-real 16.0)
@@ -1922,7 +1914,6 @@ struct WilsonEngine {
     return full ? eo_schur<18, false>(which) : eo_schur<12, false>(which);
   }
   hp_status eo_exact() {
-    dim3 gr = eo_grid();
     {
       ProfScope ps(ctx, PX == PR64 ? "k_eo_x1<fp64>" : "k_eo_x1<ff>");
       k_eo_x1<PX, NT><<<tile_grid(), NT, 0, ctx->stream>>>(a, nslots);
@@ -1989,7 +1980,6 @@ struct WilsonEngine {
       }
       HP_LAUNCH_CHECK();
       if (SPR != PR64) {
-        const dim3 gr = eo_grid();
         {
           ProfScope ps(ctx, "k_eo_src");
           k_eo_src<NT><<<tile_grid(), NT, 0, ctx->stream>>>(a, nslots);
@@ -2390,9 +2380,6 @@ static hp_status bench_wilson_t(hp_ctx* ctx, const LatGeom& g, int nrhs, int ite
   *ms = (double)t / iters;
   return HP_OK;
 }
-
-// generic slot scheduler shared by both operator families
-#include "hp_schedule.cuh"
 
 // generic slot scheduler shared by both operator families
 #include "hp_schedule.cuh"
