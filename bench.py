@@ -69,11 +69,11 @@ def source_hash(kernel):
 
 
 # DRAM traffic of the dominant kernel per byte of algorithmic work, from one ncu capture of the
-# same kernel (k_eo2_even, the two-right-hand-side even-site stencil, eo_kernel 4) on 32^3x16 with
-# 12 slots: 282.3 MB read + 143.3 MB written per launch against 377.5 MB algorithmic (12-real links;
+# same kernel (k_eo2_even, the two-right-hand-side even-site stencil, eo_kernel 4 and 5) on 32^3x16 with
+# 12 slots: 280.8 MB read + 141.7 MB written per launch against 377.5 MB algorithmic (12-real links;
 # both parts of the launch -- spinors and links -- grow with the units processed, so the ratio
 # carries over to the 32^3x64 launch); valid only for the kernel source it was taken on
-NCU_TRAFFIC = {("k_eo_even", "f7f32fc9b7f5"): {"bytes_all_slots": 282.3e6 + 143.3e6,
+NCU_TRAFFIC = {("k_eo_even", "bec4e86cbb47"): {"bytes_all_slots": 280.8e6 + 141.7e6,
                                       "alg_bytes_all_slots": 262144 * 104 * 12 + 4 * 524288 * 24}}
 
 
@@ -171,7 +171,7 @@ def kernel_bytes(name, prec, V, c):
     iterations), launches (of this kernel), exact (true-residual evaluations, including the
     initial one), groups (FP32 group updates), eo (iterating on the odd half)."""
     S, L, E = spinor_link_bytes(prec)
-    X = 192                                   # FP64 or float-float solution, per site
+    X = 192                                   # FP64 or block fixed-point solution, per site
     n, it, la = c["eo"], c["rhs_iters"], c["launches"]
     Vf = V // 2 if n else V                   # sites of the iterated vectors
     links = 4 * V * L * la

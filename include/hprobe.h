@@ -163,7 +163,12 @@ hp_status hp_probe_sequence(hp_ctx* ctx, const hp_lattice* lat, int32_t kind, in
 
 typedef struct {
     int32_t precision;      /* hp_precision                                              */
-    int32_t rhs_block;      /* right-hand sides solved concurrently (0: automatic)       */
+    int32_t rhs_block;      /* right-hand sides solved concurrently (0: automatic -- Wilson: up to 256 while their
+                               vectors take no more than 8 GB and half of the free device memory, else 4M
+                               sites' worth, so the grouping and the last bits follow the memory that is free;
+                               Laplacian: a solve per thread-block cluster where that is faster, with at most
+                               1 GB or a 32nd of the device's memory of vectors, else 4M sites' worth; the
+                               workspace stays with the context)                         */
     int32_t maxiter;        /* iterations per right-hand side (0: 10000)                 */
     int32_t dilution;       /* 12 for Wilson (full spin-colour dilution), 1 for Laplacian; 0: default */
     uint64_t z0_seed;       /* bias-removal vector, 0 = none (Section 4)                 */

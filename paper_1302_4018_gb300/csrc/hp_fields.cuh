@@ -656,11 +656,11 @@ __device__ __forceinline__ int sel4(const int (&v)[4], int mu) {
 // The sums run in integers: a link element is 2^-30 (i + l) (30-bit integer and FP32 remainder, prepared once), so the
 // product of the integer parts is one 32 x 32 + 64 bit multiply-add, exact, and only the cross terms i l + l i need FP32
 // (two FMAs, exact to 2^-24 of 2^-28).  That is 3 instructions (4 slots of the FMA pipe) per real multiply-add,
-// 32 of them per clock and SM, where float-float sums take 12 (7.8 per clock and SM); projections and reconstructions
+// 34 of them per clock and SM, where float-float sums take 12 (8.2 per clock and SM); projections and reconstructions
 // are integer adds.  The terms of a direction are shifted to the largest unit of the eight neighbours; the sums stay
-// below 2^63: |i| <= 2^28 after the projection, a row of U has norm 1, so a term is at most sqrt(6) 2^58 and eight of
-// them 2^62.3.  One conversion to float-float per result.
-// 32^3x64, per right-hand side and launch: x_1 0.43 ms, x_2 0.62 ms (float-float sums: 0.59, 0.73 ms).
+// below 2^63: |i| <= 2^28 after the projection, a row of U has norm 1 (special unitary links, as the interface asks), so a
+// term is at most sqrt(6) 2^58 and eight of them 2^62.3.  One conversion to float-float per result.
+// 32^3x64, per right-hand side and launch: x_1 0.43 ms, x_2 0.57 ms (float-float sums: 0.59, 0.73 ms).
 // The directions run in a loop that is not unrolled, with one copy of the SU(3) product for all of them (a backward link
 // enters as its adjoint, formed in registers): unrolled, eight copies overflow the instruction cache.
 template <int SPR, int LPR, int REC, bool HALF>

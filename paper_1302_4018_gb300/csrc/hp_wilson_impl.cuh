@@ -913,7 +913,7 @@ __global__ void __launch_bounds__(NT) k_bicg_p(WArgs a) {
 }
 
 // ---- harvest: q = v^H x = sum_site conj(v(site)) x(site, a)   (FP64)
-// one component of the converged solution in FP64 (from FP64 or float-float storage)
+// one component of the converged solution in FP64 (from FP64 or block fixed-point storage)
 __device__ __forceinline__ double2 solution_component(const WArgs& a, int slot, int site, int comp) {
   if (a.x) return a.x[((size_t)slot * 12 + comp) * a.Vmax + site];
   return SpinorIO<PRFF>::component(a.xff, a.Vmax, slot, site, comp);
@@ -1201,7 +1201,7 @@ __global__ void __launch_bounds__(NT, EO_ODD_MINB(SIN, REC)) k_eo_odd(WArgs a, F
 }
 
 // the exact steps: resident blocks of 128 threads (register caps, chosen by timing on 32^3x64):
-// step 1 at 3 (168 registers), the float-float step 2 at 2 (its hop plus the residual epilogue
+// step 1 at 3 (168 registers), the 48-bit step 2 at 2 (its hop plus the residual epilogue
 // spills at 168; without spills it runs 13% faster)
 #define EO_X_MINB 3
 #define EO_X2_MINB 2
@@ -1547,7 +1547,7 @@ static __global__ void k_eo_grad(WArgs a, int lat, const int* __restrict__ slots
 }
 
 // ---- the solutions of harvested slots in the canonical layout: slot slots[i] -> right-hand side idx[i]
-// of out (complex [n][V][12]; FP64, float-float hi + lo, or the two parities of the even-odd iteration)
+// of out (complex [n][V][12]; from FP64 or block fixed point, whole or the two parities of the even-odd iteration)
 static __global__ void k_w_keep(WArgs a, const int* __restrict__ slots, const int* __restrict__ idx, int nsl,
                                 double2* __restrict__ out, LatGeom g) {
   const long long total = (long long)nsl * g.V;
@@ -1637,7 +1637,7 @@ struct WilsonEngine {
         HP_TRY(hp_ws(ctx, "solve.xe", sizeof(double2) * 12 * (size_t)ns * Vmax, &p));
         a.xe = (double2*)p;
       }
-    } else {   // float-float solution
+    } else {   // solution in block fixed point
       HP_TRY(alloc_field(ctx, "solve.xhi", PR32, ns, Vmax, &a.xff));   // integers
       FieldPtr lo;
       HP_TRY(alloc_field(ctx, "solve.xlo", PR32, ns, Vmax, &lo));      // remainders
